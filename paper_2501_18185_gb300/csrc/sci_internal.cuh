@@ -88,6 +88,8 @@ struct RefW {
 // up to 4,489 (140 spin-orbitals) 25.8 ms at 2048, 20.2 ms at 512; a space whose buckets
 // stay below 512 (30 orbitals, up to 441) is unchanged, and tiling it at 256 costs 2%.
 constexpr int kTileBucket = 512;
+constexpr int kSortBucket = 64;     // buckets of at most this many members go through the sorted kernel
+constexpr int kSmallBucket = 4;     // ... and of at most this many through the register kernel
 constexpr int kTileRows = 256;      // rows of a tile of the tiled kernel (one per thread)
 // launches that stage 64 bytes or more per window row (8 real vectors) tile from this
 // size instead (measured on the 30-orbital 2M space, buckets up to 441: FP64 x 8
@@ -107,6 +109,7 @@ struct Split {
 struct TileSplit {
     uint32_t *tiles = nullptr;
     Split base, wide;
+    int64_t above[kSortBucket + 1] = {};   // entries [0, above[s]) are the buckets of more than s members
 };
 // whether two members of a bucket share an extra orbital (then they are a single
 // excitation of each other, not a double); valid for orbitals up to 255

@@ -693,19 +693,25 @@ int order_runs(sci_ctx *ctx, int nruns, Buckets &B)
     return SCI_OK;
 }
 
-// ------------------------------------------------------------------ tiled prefix
-// The (N-2) table holds its buckets largest first, so the buckets of more than thr
-// members are its first entries.  out[0] = the end of that prefix (written by the one
-// entry where the sizes cross thr); out[1] counts entries where a bucket above thr follows
-// one at or below it, which a table in size order never has.
-__global__ void k_split_point(const uint32_t *__restrict__ e_pos, int64_t E, int thr, unsigned long long *out)
+// ------------------------------------------------------------------ size bounds
+// The (N-2) table holds its buckets largest first, so the buckets of more than thr members
+// are its first entries.  Thread t finds the end of that prefix for its threshold by
+// bisection: out[t], and the bucket size found there (0 at the end of the table) in out[n + t].
+struct Thresholds {
+    int n, thr[sci::kSortBucket + 3];
+};
+__global__ void k_size_bounds(const uint32_t *__restrict__ e_pos, int64_t E, Thresholds q, int64_t *__restrict__ out)
 {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < E; p += (int64_t)gridDim.x * blockDim.x) {
-        const bool big = sci::pos_size(e_pos[p]) > thr;
-        const bool next_big = p + 1 < E && sci::pos_size(e_pos[p + 1]) > thr;
-        if (big && !next_big) out[0] = (unsigned long long)(p + 1);
-        if (!big && next_big) atomicAdd(out + 1, 1ull);
+    const int t = threadIdx.x;
+    if (t >= q.n) return;
+    int64_t lo = 0, hi = E;   // every entry below lo is above the threshold, every one from hi on is not
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (sci::pos_size(e_pos[mid]) > q.thr[t]) lo = mid + 1;
+        else hi = mid;
     }
+    out[t] = lo;
+    out[q.n + t] = lo < E ? sci::pos_size(e_pos[lo]) : 0;
 }
 
 // tile starts: the entries at bucket offsets 0, kTileRows, 2 kTileRows, ...
@@ -731,32 +737,6 @@ void sci_free_split(sci_ctx *ctx, bool ranged)
     sp = sci::TileSplit{};
 }
 
-namespace {
-// the split at threshold thr: the end of the prefix of buckets above thr and the largest
-// bucket after it
-int split_point(sci_ctx *ctx, const uint32_t *e_pos, int64_t E, int thr, sci::Split &out)
-{
-    cudaStream_t st = ctx->stream;
-    TmpBuf cnt;
-    unsigned long long h[2] = {0, 0};
-    SCI_CK(cudaMalloc(&cnt.p, 16));
-    SCI_CK(cudaMemsetAsync(cnt.p, 0, 16, st));
-    k_split_point<<<grid_for(E), 256, 0, st>>>(e_pos, E, thr, cnt.as<unsigned long long>());
-    SCI_CK(cudaGetLastError());
-    SCI_CK(cudaMemcpyAsync(h, cnt.p, 16, cudaMemcpyDeviceToHost, st));
-    SCI_CK(cudaStreamSynchronize(st));
-    if (h[1] != 0) return sci_fail(ctx, SCI_ERR_STATE, "internal: (N-2) buckets not in size order");
-    out.big = (int64_t)h[0];
-    out.maxb_small = 0;
-    if (out.big < E) {
-        uint32_t pos = 0;
-        SCI_CK(cudaMemcpy(&pos, e_pos + out.big, 4, cudaMemcpyDeviceToHost));
-        out.maxb_small = sci::pos_size(pos);
-    }
-    return SCI_OK;
-}
-}  // namespace
-
 int sci_table_split(sci_ctx *ctx, bool ranged)
 {
     sci_free_split(ctx, ranged);
@@ -766,9 +746,22 @@ int sci_table_split(sci_ctx *ctx, bool ranged)
     cudaStream_t st = ctx->stream;
     sci::TileSplit sp;
     const int thr_wide = ctx->tile_user ? ctx->tile_b : std::min(ctx->tile_b, sci::kTileBucketWide);
-    int rc = split_point(ctx, e_pos, E, ctx->tile_b, sp.base);
-    if (rc == SCI_OK) rc = split_point(ctx, e_pos, E, thr_wide, sp.wide);
-    if (rc != SCI_OK) return rc;
+    Thresholds q;
+    q.n = sci::kSortBucket + 3;
+    q.thr[0] = ctx->tile_b, q.thr[1] = thr_wide;
+    for (int k = 0; k <= sci::kSortBucket; k++) q.thr[2 + k] = k;
+    int64_t h[2 * (sci::kSortBucket + 3)];
+    {
+        TmpBuf out;
+        SCI_CK(cudaMalloc(&out.p, sizeof h));
+        k_size_bounds<<<1, 96, 0, st>>>(e_pos, E, q, out.as<int64_t>());
+        SCI_CK(cudaGetLastError());
+        SCI_CK(cudaMemcpyAsync(h, out.p, sizeof h, cudaMemcpyDeviceToHost, st));
+        SCI_CK(cudaStreamSynchronize(st));
+    }
+    sp.base.big = h[0], sp.base.maxb_small = (int)h[q.n];
+    sp.wide.big = h[1], sp.wide.maxb_small = (int)h[q.n + 1];
+    for (int k = 0; k <= sci::kSortBucket; k++) sp.above[k] = h[2 + k];
     const int64_t big = sp.wide.big;   // >= sp.base.big: the lower threshold tiles more
     if (big > 0) {
         TmpBuf flag, at, tmp;

@@ -18,16 +18,19 @@
 // (the closed-shell reference simplification of Sec. 2.3).
 //
 // Kernel shape (bucket-major, no tensor cores: this is a sparse gather).  A CTA owns
-// the whole buckets that start in its range of CH table rows (its window), and stages
-// every member of them in shared memory: the member's ket code, its ket offset into the
-// pair-integral table and its coefficients pre-multiplied by (-1)^pi.  Each thread owns
-// a row and walks the members of its bucket (in the FP64 kernels, the members other than
-// the row itself); lanes of a warp that share a bucket read the same member, or one of
-// two neighbours (a shared-memory broadcast), and nearby pair-table entries (the table
-// stores bra indices fastest).  A row's partial sum is added to sigma with one FP64
-// atomic add per (bucket, member).  Buckets too large to stage beside a window (above
-// the tile threshold) are walked by k_doubles_tiled instead: 256 members of one bucket as
-// the rows of a CTA, the whole bucket streamed through shared memory in column tiles.
+// the whole buckets that start in its range of table rows (its window), and stages every
+// member of them in shared memory: the member's ket code, its ket offset into the
+// pair-integral table and its coefficients pre-multiplied by (-1)^pi.  A thread takes a row
+// and the members of its bucket that are doubles of it; the table stores bra indices
+// fastest, so lanes that share a bucket read nearby entries.  A row's partial sum is added
+// to sigma with one FP64 atomic add per (bucket, member).  Three things bound it, in turn:
+// the FP64 pipe (2 FMA per clock per SM: a warp instruction holds it 16 cycles whatever its
+// active lanes), the L1's rate of scattered accesses and the latency of the L2 gathers.
+// Buckets are handled by size (launch_doubles): above the tile threshold by
+// k_doubles_tiled, 256 members of one bucket as the rows of a CTA and the bucket streamed
+// through shared memory; then by k_doubles_aligned (lanes of a bucket in step) or
+// k_doubles_sorted (rows sorted by their number of doubles, lanes on useful products only);
+// the smallest by k_doubles_small, in registers.
 #include <algorithm>
 #include <cstdio>
 #include <vector>
@@ -37,6 +40,12 @@
 #include "sci_internal.cuh"
 
 using sci::zdbl;
+
+#define SCI_CK(call)                                                 \
+    do {                                                             \
+        int _rc = sci_cuda_check(ctx, (call), #call);                \
+        if (_rc != SCI_OK) return _rc;                               \
+    } while (0)
 
 namespace {
 
@@ -91,6 +100,8 @@ template <> __device__ __forceinline__ zdbl ldg<zdbl>(const zdbl *p)
 }
 
 using sci::col_code;
+using sci::kSmallBucket;
+using sci::kSortBucket;
 using sci::disjoint;
 using sci::row_code;
 using sci::window;
@@ -176,103 +187,6 @@ __global__ void k_sigma_init(const double *__restrict__ hdiag, const TC *__restr
     }
 }
 
-// ------------------------------------------------------------------ doubles (FP64)
-// TS: storage type of tab and staged coefficients; TA: accumulator (FP64 / complex128).
-// Shared memory per staged member: (ket code, ket table offset) as uint2, and its NV
-// coefficients times (-1)^pi.
-template <typename TS, typename TC, int NV, bool RANGED, bool STORE = false>
-__global__ void __launch_bounds__(kThreads)
-k_doubles(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict__ e_code, const uint32_t *__restrict__ e_pos,
-          int64_t E, int CH, sci::TabRule tr, const TS *__restrict__ tab, const TC *__restrict__ C, int nvec, int v0,
-          typename AccOf<TS>::type *__restrict__ Sout, sci::RowRange rr, const uint32_t *__restrict__ slot)
-{
-    using TA = typename AccOf<TS>::type;
-    extern __shared__ __align__(16) unsigned char smem[];
-    int64_t r0, r1;
-    window(e_pos, E, CH, r0, r1);
-    if (r0 >= r1) return;
-    const int W = (int)(r1 - r0);
-    TS *s_c = reinterpret_cast<TS *>(smem);
-    const size_t cbytes = ((size_t)W * NV * sizeof(TS) + 15) & ~(size_t)15;
-    uint2 *s_kc = reinterpret_cast<uint2 *>(smem + cbytes);
-    uint16_t *s_own = reinterpret_cast<uint16_t *>(smem + cbytes + (size_t)W * sizeof(uint2));
-    int nrows = W;
-    if constexpr (RANGED) {
-        nrows = owned_rows(e_idx, r0, W, rr, s_own);
-        if (nrows == 0) return;
-    }
-
-    for (int q = threadIdx.x; q < W; q += blockDim.x) {
-        const int64_t g = r0 + q;
-        const uint32_t idx = e_idx[g], code = e_code[g];
-        uint32_t rowoff, colbase;
-        sci::pair_offsets(tr, sci::code_x(code), sci::code_y(code), rowoff, colbase);
-        s_kc[q] = make_uint2(col_code(code), colbase);
-        const bool par = sci::code_par(code);
-#pragma unroll
-        for (int v = 0; v < NV; v++) s_c[q * NV + v] = flip(par, (TS)C[(int64_t)idx * nvec + v0 + v]);
-    }
-    __syncthreads();
-
-    for (int t_ = threadIdx.x; t_ < nrows; t_ += blockDim.x) {
-        const int q0 = RANGED ? (int)s_own[t_] : t_;
-        const uint32_t code = e_code[r0 + q0], pos = e_pos[r0 + q0];
-        uint32_t rowoff, colbase;
-        sci::pair_offsets(tr, sci::code_x(code), sci::code_y(code), rowoff, colbase);
-        const int bs = q0 - sci::pos_off(pos), je = bs + sci::pos_size(pos) - 1;
-        const uint32_t rc = row_code(code);
-        const TS *trow = tab + rowoff;
-        TA acc[NV];
-#pragma unroll
-        for (int v = 0; v < NV; v++) zero(acc[v]);
-        // the members other than the row itself: j in [bs, je) stands for bucket position
-        // j + (j >= q0), so rows of equal bucket size (windows hold buckets of one size,
-        // largest first) run the same trip count and no FP64 FMA is spent on the row (one
-        // in 3.5 members on average).  Groups of kUnroll members: a group with no double
-        // of this row (single excitations of it) is skipped, and so is the whole warp's
-        // work when no lane has one; otherwise up to kUnroll table loads are in flight per
-        // thread and a non-double member contributes t = 0
-        int j = bs;
-        for (; j + kUnroll <= je; j += kUnroll) {
-            uint2 kc[kUnroll];
-            TS t[kUnroll];
-            unsigned vm = 0;
-#pragma unroll
-            for (int u = 0; u < kUnroll; u++) {
-                kc[u] = s_kc[j + u + (j + u >= q0)];
-                vm |= (unsigned)disjoint(rc, kc[u].x) << u;
-            }
-            if (vm == 0) continue;
-#pragma unroll
-            for (int u = 0; u < kUnroll; u++) {
-                zero(t[u]);
-                if (vm & (1u << u)) t[u] = ldg(trow + kc[u].y);
-            }
-#pragma unroll
-            for (int u = 0; u < kUnroll; u++)
-#pragma unroll
-                for (int v = 0; v < NV; v++) fma_acc(acc[v], t[u], s_c[(j + u + (j + u >= q0)) * NV + v]);
-        }
-        for (; j < je; j++) {
-            const int m = j + (j >= q0);
-            const uint2 kc = s_kc[m];
-            if (!disjoint(rc, kc.x)) continue;
-            const TS t = ldg(trow + kc.y);
-#pragma unroll
-            for (int v = 0; v < NV; v++) fma_acc(acc[v], t, s_c[m * NV + v]);
-        }
-        const bool par = sci::code_par(code);
-        if constexpr (STORE) {   // the row sum to this entry's slot (summed per row later)
-#pragma unroll
-            for (int v = 0; v < NV; v++) Sout[(int64_t)slot[r0 + q0] * nvec + v0 + v] = flip(par, acc[v]);
-        } else {
-            const uint32_t idx = e_idx[r0 + q0];
-#pragma unroll
-            for (int v = 0; v < NV; v++) red_add(Sout + (int64_t)idx * nvec + v0 + v, flip(par, acc[v]));
-        }
-    }
-}
-
 // ------------------------------------------------------------------ doubles, paired FP32
 // The same bucket walk with the products and per-row sums in "double-single" arithmetic
 // on the FP32 pipes: an FP64 value x is carried as hi + lo with hi = fl32(x) and
@@ -320,97 +234,6 @@ __device__ __forceinline__ void ds_fma1(Ds &a, float t, float c)
     a.hi = s;
 }
 
-// FP32 storage: the pair table rounded to FP32 (tab32) and FP32 coefficients, exact
-// products, compensated bucket sums, FP64 accumulation into sigma
-template <int NV, bool RANGED, bool STORE = false>
-__global__ void __launch_bounds__(kThreads, NV >= 8 ? SCI_F32_MINB : 1)
-k_doubles_f32(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict__ e_code,
-              const uint32_t *__restrict__ e_pos, int64_t E, int CH, sci::TabRule tr,
-              const float *__restrict__ tab32, const float *__restrict__ C, int nvec, int v0,
-              double *__restrict__ Sout, sci::RowRange rr, const uint32_t *__restrict__ slot)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    int64_t r0, r1;
-    window(e_pos, E, CH, r0, r1);
-    if (r0 >= r1) return;
-    const int W = (int)(r1 - r0);
-    float *s_c = reinterpret_cast<float *>(smem);
-    const size_t cbytes = ((size_t)W * NV * sizeof(float) + 15) & ~(size_t)15;
-    uint2 *s_kc = reinterpret_cast<uint2 *>(smem + cbytes);
-    uint16_t *s_own = reinterpret_cast<uint16_t *>(smem + cbytes + (size_t)W * sizeof(uint2));
-    int nrows = W;
-    if constexpr (RANGED) {
-        nrows = owned_rows(e_idx, r0, W, rr, s_own);
-        if (nrows == 0) return;
-    }
-
-    for (int q = threadIdx.x; q < W; q += blockDim.x) {
-        const int64_t g = r0 + q;
-        const uint32_t idx = e_idx[g], code = e_code[g];
-        uint32_t rowoff, colbase;
-        sci::pair_offsets(tr, sci::code_x(code), sci::code_y(code), rowoff, colbase);
-        s_kc[q] = make_uint2(col_code(code), colbase);
-        const bool par = sci::code_par(code);
-#pragma unroll
-        for (int v = 0; v < NV; v++) s_c[q * NV + v] = flip(par, C[(int64_t)idx * nvec + v0 + v]);
-    }
-    __syncthreads();
-
-    for (int t_ = threadIdx.x; t_ < nrows; t_ += blockDim.x) {
-        const int q0 = RANGED ? (int)s_own[t_] : t_;
-        const uint32_t code = e_code[r0 + q0], pos = e_pos[r0 + q0];
-        uint32_t rowoff, colbase;
-        sci::pair_offsets(tr, sci::code_x(code), sci::code_y(code), rowoff, colbase);
-        const int bs = q0 - sci::pos_off(pos), be = bs + sci::pos_size(pos);
-        const uint32_t rc = row_code(code);
-        const float *trow = tab32 + rowoff;
-        Ds acc[NV];
-#pragma unroll
-        for (int v = 0; v < NV; v++) ds_zero(acc[v]);
-        // all members, the row itself included (t = 0): this kernel is bound by its FP64
-        // atomics, and the aligned walk keeps lanes of one bucket on the same member
-        int j = bs;
-        for (; j + kUnroll <= be; j += kUnroll) {
-            uint2 kc[kUnroll];
-            float t[kUnroll];
-            unsigned vm = 0;
-#pragma unroll
-            for (int u = 0; u < kUnroll; u++) {
-                kc[u] = s_kc[j + u];
-                vm |= (unsigned)disjoint(rc, kc[u].x) << u;
-            }
-            if (vm == 0) continue;
-#pragma unroll
-            for (int u = 0; u < kUnroll; u++) {
-                t[u] = 0.f;
-                if (vm & (1u << u)) t[u] = __ldg(trow + kc[u].y);
-            }
-#pragma unroll
-            for (int u = 0; u < kUnroll; u++)
-#pragma unroll
-                for (int v = 0; v < NV; v++) ds_fma1(acc[v], t[u], s_c[(j + u) * NV + v]);
-#pragma unroll
-            for (int v = 0; v < NV; v++) ds_renorm(acc[v]);
-        }
-        for (; j < be; j++) {
-            const uint2 kc = s_kc[j];
-            if (!disjoint(rc, kc.x)) continue;
-            const float t = __ldg(trow + kc.y);
-#pragma unroll
-            for (int v = 0; v < NV; v++) ds_fma1(acc[v], t, s_c[j * NV + v]);
-        }
-        const bool par = sci::code_par(code);
-        if constexpr (STORE) {
-#pragma unroll
-            for (int v = 0; v < NV; v++) Sout[(int64_t)slot[r0 + q0] * nvec + v0 + v] = flip(par, ds_value(acc[v]));
-        } else {
-            const uint32_t idx = e_idx[r0 + q0];
-#pragma unroll
-            for (int v = 0; v < NV; v++) red_add_nz(Sout + (int64_t)idx * nvec + v0 + v, flip(par, ds_value(acc[v])));
-        }
-    }
-}
-
 __global__ void k_split_cz(const zdbl *__restrict__ C, int64_t M, int nvec, int v0, int G, float4 *__restrict__ out)
 {
     const int64_t total = M * G;
@@ -421,192 +244,53 @@ __global__ void k_split_cz(const zdbl *__restrict__ C, int64_t M, int nvec, int 
     }
 }
 
-// real: tab2 is the (hi, lo) split of the pair table, C2 the split vector group
-template <int NV, bool RANGED, bool STORE = false>
-__global__ void __launch_bounds__(kThreads)
-k_doubles_ds(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict__ e_code,
-             const uint32_t *__restrict__ e_pos, int64_t E, int CH, sci::TabRule tr,
-             const float2 *__restrict__ tab2, const float2 *__restrict__ C2, int nvec, int v0,
-             double *__restrict__ Sout, sci::RowRange rr, const uint32_t *__restrict__ slot)
+// ------------------------------------------------------------------ chained launches
+// The doubles launches of one vector group, and in FP64 those of all groups and the singles,
+// only read what was complete before the first of them and add into sigma (or store to slots
+// of their own), so each may start while its predecessor drains: a dependent launch
+// (programmatic stream serialization) begins once every CTA of the predecessor has started
+// and executed chain_next().  A later launch must still see all of them complete, so a launch
+// completes only after its predecessor: its last CTA (the singles: every CTA, at its end) does
+// nothing but wait for it.  A selected space takes seven of these launches, the first of them
+// over few, long rows, and its drain is what the chain fills: 60k-determinant 30-orbital space
+// 429 us launched one after another, 336 chained; 64 spinors, M = 500k 8.85 -> 8.66 ms; full CI
+// of 10 orbitals with 4 + 2 electrons, three vectors 117 -> 71 us.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// at the start of a chained kernel, launched with one CTA more than it has work for: true in
+// that CTA, once the predecessor has completed
+__device__ __forceinline__ bool chain_last_cta()
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    int64_t r0, r1;
-    window(e_pos, E, CH, r0, r1);
-    if (r0 >= r1) return;
-    const int W = (int)(r1 - r0);
-    float2 *s_c = reinterpret_cast<float2 *>(smem);
-    const size_t cbytes = ((size_t)W * NV * sizeof(float2) + 15) & ~(size_t)15;
-    uint2 *s_kc = reinterpret_cast<uint2 *>(smem + cbytes);
-    uint16_t *s_own = reinterpret_cast<uint16_t *>(smem + cbytes + (size_t)W * sizeof(uint2));
-    int nrows = W;
-    if constexpr (RANGED) {
-        nrows = owned_rows(e_idx, r0, W, rr, s_own);
-        if (nrows == 0) return;
-    }
-
-    for (int q = threadIdx.x; q < W; q += blockDim.x) {
-        const int64_t g = r0 + q;
-        const uint32_t idx = e_idx[g], code = e_code[g];
-        uint32_t rowoff, colbase;
-        sci::pair_offsets(tr, sci::code_x(code), sci::code_y(code), rowoff, colbase);
-        s_kc[q] = make_uint2(col_code(code), colbase);
-        const bool par = sci::code_par(code);
-#pragma unroll
-        for (int v = 0; v < NV; v++) s_c[q * NV + v] = flip(par, C2[(int64_t)idx * NV + v]);
-    }
-    __syncthreads();
-
-    for (int t_ = threadIdx.x; t_ < nrows; t_ += blockDim.x) {
-        const int q0 = RANGED ? (int)s_own[t_] : t_;
-        const uint32_t code = e_code[r0 + q0], pos = e_pos[r0 + q0];
-        uint32_t rowoff, colbase;
-        sci::pair_offsets(tr, sci::code_x(code), sci::code_y(code), rowoff, colbase);
-        const int bs = q0 - sci::pos_off(pos), be = bs + sci::pos_size(pos);
-        const uint32_t rc = row_code(code);
-        const float2 *trow = tab2 + rowoff;
-        Ds acc[NV];
-#pragma unroll
-        for (int v = 0; v < NV; v++) ds_zero(acc[v]);
-        // all members, the row itself included (it contributes t = 0): lanes of one bucket
-        // then read the same member and neighbouring table entries at every step, which
-        // this LSU-bound kernel needs more than the skipped arithmetic
-        int j = bs;
-        for (; j + kUnroll <= be; j += kUnroll) {
-            uint2 kc[kUnroll];
-            float2 t[kUnroll];
-            unsigned vm = 0;
-#pragma unroll
-            for (int u = 0; u < kUnroll; u++) {
-                kc[u] = s_kc[j + u];
-                vm |= (unsigned)disjoint(rc, kc[u].x) << u;
-            }
-            if (vm == 0) continue;
-#pragma unroll
-            for (int u = 0; u < kUnroll; u++) {
-                t[u] = make_float2(0.f, 0.f);
-                if (vm & (1u << u)) t[u] = __ldg(trow + kc[u].y);
-            }
-#pragma unroll
-            for (int u = 0; u < kUnroll; u++)
-#pragma unroll
-                for (int v = 0; v < NV; v++) ds_fma(acc[v], t[u], s_c[(j + u) * NV + v]);
-#pragma unroll
-            for (int v = 0; v < NV; v++) ds_renorm(acc[v]);
-        }
-        for (; j < be; j++) {
-            const uint2 kc = s_kc[j];
-            if (!disjoint(rc, kc.x)) continue;
-            const float2 t = __ldg(trow + kc.y);
-#pragma unroll
-            for (int v = 0; v < NV; v++) ds_fma(acc[v], t, s_c[j * NV + v]);
-        }
-        const bool par = sci::code_par(code);
-        if constexpr (STORE) {
-#pragma unroll
-            for (int v = 0; v < NV; v++) Sout[(int64_t)slot[r0 + q0] * nvec + v0 + v] = flip(par, ds_value(acc[v]));
-        } else {
-            const uint32_t idx = e_idx[r0 + q0];
-#pragma unroll
-            for (int v = 0; v < NV; v++) red_add(Sout + (int64_t)idx * nvec + v0 + v, flip(par, ds_value(acc[v])));
-        }
-    }
+    chain_next();
+    if (blockIdx.x != gridDim.x - 1) return false;
+    chain_wait();
+    return true;
 }
 
-// complex: tab4 holds (re_hi, re_lo, im_hi, im_lo); C4 the split vector group
-template <int NV, bool RANGED, bool STORE = false>
-__global__ void __launch_bounds__(kThreads)
-k_doubles_dsz(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict__ e_code,
-              const uint32_t *__restrict__ e_pos, int64_t E, int CH, sci::TabRule tr,
-              const float4 *__restrict__ tab4, const float4 *__restrict__ C4, int nvec, int v0, zdbl *__restrict__ Sout,
-              sci::RowRange rr, const uint32_t *__restrict__ slot)
+template <typename... K, typename... A>
+cudaError_t launch_chained(bool dependent, void (*kern)(K...), dim3 grid, size_t smem, cudaStream_t st, A... args)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    int64_t r0, r1;
-    window(e_pos, E, CH, r0, r1);
-    if (r0 >= r1) return;
-    const int W = (int)(r1 - r0);
-    float4 *s_c = reinterpret_cast<float4 *>(smem);
-    const size_t cbytes = ((size_t)W * NV * sizeof(float4) + 15) & ~(size_t)15;
-    uint2 *s_kc = reinterpret_cast<uint2 *>(smem + cbytes);
-    uint16_t *s_own = reinterpret_cast<uint16_t *>(smem + cbytes + (size_t)W * sizeof(uint2));
-    int nrows = W;
-    if constexpr (RANGED) {
-        nrows = owned_rows(e_idx, r0, W, rr, s_own);
-        if (nrows == 0) return;
-    }
-
-    for (int q = threadIdx.x; q < W; q += blockDim.x) {
-        const int64_t g = r0 + q;
-        const uint32_t idx = e_idx[g], code = e_code[g];
-        uint32_t rowoff, colbase;
-        sci::pair_offsets(tr, sci::code_x(code), sci::code_y(code), rowoff, colbase);
-        s_kc[q] = make_uint2(col_code(code), colbase);
-        const bool par = sci::code_par(code);
-#pragma unroll
-        for (int v = 0; v < NV; v++) s_c[q * NV + v] = flip(par, C4[(int64_t)idx * NV + v]);
-    }
-    __syncthreads();
-
-    for (int t_ = threadIdx.x; t_ < nrows; t_ += blockDim.x) {
-        const int q0 = RANGED ? (int)s_own[t_] : t_;
-        const uint32_t code = e_code[r0 + q0], pos = e_pos[r0 + q0];
-        uint32_t rowoff, colbase;
-        sci::pair_offsets(tr, sci::code_x(code), sci::code_y(code), rowoff, colbase);
-        const int bs = q0 - sci::pos_off(pos), je = bs + sci::pos_size(pos) - 1;
-        const uint32_t rc = row_code(code);
-        const float4 *trow = tab4 + rowoff;
-        Ds ar[NV], ai[NV];
-#pragma unroll
-        for (int v = 0; v < NV; v++) ds_zero(ar[v]), ds_zero(ai[v]);
-        int nused = 0;
-        // the members other than the row itself (bucket position j + (j >= q0))
-        for (int j = bs; j < je; j++) {
-            const int m = j + (j >= q0);
-            const uint2 kc = s_kc[m];
-            if (!disjoint(rc, kc.x)) continue;
-            const float4 t = __ldg(trow + kc.y);
-            const float2 tr_ = make_float2(t.x, t.y), ti = make_float2(t.z, t.w);
-            const float2 mti = make_float2(-t.z, -t.w);
-#pragma unroll
-            for (int v = 0; v < NV; v++) {
-                const float4 c = s_c[m * NV + v];
-                const float2 cr = make_float2(c.x, c.y), ci = make_float2(c.z, c.w);
-                ds_fma(ar[v], tr_, cr);
-                ds_fma(ar[v], mti, ci);
-                ds_fma(ai[v], tr_, ci);
-                ds_fma(ai[v], ti, cr);
-            }
-            if ((++nused & 3) == 0)
-#pragma unroll
-                for (int v = 0; v < NV; v++) ds_renorm(ar[v]), ds_renorm(ai[v]);
-        }
-        const bool par = sci::code_par(code);
-        if constexpr (STORE) {
-#pragma unroll
-            for (int v = 0; v < NV; v++)
-                Sout[(int64_t)slot[r0 + q0] * nvec + v0 + v] = flip(par, zdbl{ds_value(ar[v]), ds_value(ai[v])});
-        } else {
-            const uint32_t idx = e_idx[r0 + q0];
-#pragma unroll
-            for (int v = 0; v < NV; v++)
-                red_add(Sout + (int64_t)idx * nvec + v0 + v, flip(par, zdbl{ds_value(ar[v]), ds_value(ai[v])}));
-        }
-    }
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, (K)args...);
 }
 
-// ------------------------------------------------------------------ doubles, tiled
-// (N-2) buckets of more than tile_b members (sci_set_tile_threshold) are too large to
-// stage whole beside a window, so they run here.  A CTA takes kTileRows consecutive
-// members of one bucket as its rows (one per thread) and streams the bucket's members
-// through shared memory in column tiles, each staged once per CTA; every thread walks a
-// column tile against its row as the window kernels walk a bucket (disjointness test, one
-// table load per double, the FMAs), so a row sums the same products.  The row itself and
-// its single excitations fail the disjointness test and add nothing.  All threads of a
-// CTA share the bucket, so trip counts are uniform and the barriers are CTA-wide.
-// The arithmetic is a policy: staged element SC, table element TT, accumulator ACC,
-// output TO, input coefficients CI; how a coefficient is read, multiplied in,
-// renormalised (paired FP32) and written out.
-template <typename TS, typename TC> struct PolF64 {   // FP64 / complex128 (the k_doubles arithmetic)
+// ------------------------------------------------------------------ arithmetic policies
+// The arithmetic of the bucket walks is a policy: staged element SC, table element TT,
+// accumulator ACC, output TO, input coefficients CI; how a coefficient is read, multiplied
+// in, renormalised (paired FP32) and written out.
+template <typename TS, typename TC> struct PolF64 {   // FP64 / complex128
+    static constexpr bool kFp64 = true;
+    static constexpr bool kSplit = false;
+    static constexpr bool kSkipSelf = true;
     using SC = TS;
     using TT = TS;
     using ACC = typename AccOf<TS>::type;
@@ -620,7 +304,10 @@ template <typename TS, typename TC> struct PolF64 {   // FP64 / complex128 (the 
     __device__ static TO value(const ACC &a) { return a; }
     __device__ static void add_out(TO *p, TO v) { red_add(p, v); }
 };
-struct PolDS {   // paired FP32, real (the k_doubles_ds arithmetic)
+struct PolDS {   // paired FP32, real
+    static constexpr bool kFp64 = false;
+    static constexpr bool kSplit = true;
+    static constexpr bool kSkipSelf = false;
     using SC = float2;
     using TT = float2;
     using ACC = Ds;
@@ -634,7 +321,10 @@ struct PolDS {   // paired FP32, real (the k_doubles_ds arithmetic)
     __device__ static TO value(const ACC &a) { return ds_value(a); }
     __device__ static void add_out(TO *p, TO v) { red_add(p, v); }
 };
-struct PolF32 {   // FP32 storage, paired-FP32 sums (the k_doubles_f32 arithmetic)
+struct PolF32 {   // FP32 storage, paired-FP32 sums
+    static constexpr bool kFp64 = false;
+    static constexpr bool kSplit = false;
+    static constexpr bool kSkipSelf = false;
     using SC = float;
     using TT = float;
     using ACC = Ds;
@@ -652,7 +342,10 @@ __device__ __forceinline__ void PolF32::mul_add(Ds &a, float t, float c) { ds_fm
 struct DsZ {
     Ds r, i;
 };
-struct PolDSZ {   // paired FP32, complex (the k_doubles_dsz arithmetic)
+struct PolDSZ {   // paired FP32, complex
+    static constexpr bool kFp64 = false;
+    static constexpr bool kSplit = true;
+    static constexpr bool kSkipSelf = true;
     using SC = float4;
     using TT = float4;
     using ACC = DsZ;
@@ -675,10 +368,492 @@ struct PolDSZ {   // paired FP32, complex (the k_doubles_dsz arithmetic)
     __device__ static void add_out(TO *p, TO v) { red_add(p, v); }
 };
 
+// ------------------------------------------------------------------ rules by policy and width
+// the FP32-storage launch at 8 vectors
+template <class P, int NV> constexpr bool f32_wide() { return NV >= 8 && sizeof(typename P::SC) == sizeof(float); }
+
+// CTAs per SM that the bucket walks are held to: the gathers' latency asks for warps, the
+// accumulators of a wide vector group for registers.  (Left to itself the compiler takes 40
+// registers for one FP64 vector, 6 CTAs per SM.)
+template <class P, int NV> constexpr int min_ctas()
+{
+    constexpr size_t b = NV * sizeof(typename P::SC);
+    return f32_wide<P, NV>() ? SCI_F32_MINB : b <= 8 ? 8 : b <= 16 ? 6 : b <= 32 ? 5 : 4;
+}
+// ... and those of the aligned walk above kSortBucket members, whose threads walk hundreds of
+// members: more registers let it hold more table loads in flight (60k-determinant 30-orbital
+// space, one FP64 vector: 443 us at 8 CTAs, 227 at 6; 27 orbitals, two paired-FP32 vectors:
+// 278 us at 6, 155 at 5; FP32 storage at 8 vectors loses, 596 us at 5, 617 at 4)
+template <class P, int NV> constexpr int wide_ctas()
+{
+    constexpr int c = min_ctas<P, NV>();
+    return f32_wide<P, NV>() ? c : c == 8 ? 6 : c == 6 ? 5 : c;
+}
+// Window rows of that walk: `rows` or 512 when they give kWindowsWanted windows (two for
+// every resident CTA), else 256 (60k space: 85 windows of 768 rows 227 us, 254 of 256 rows 148
+// us; 40 orbitals, two vectors: 1,188 of 768 rows 1.21 ms, 3,563 of 256 1.14 ms; with 6,645
+// windows of 768 rows, on the 2M space, 256 rows cost 3%).
+constexpr int64_t kWindowsWanted = 152 * 16;
+inline int window_rows(int64_t entries, int rows)
+{
+    for (int r : {rows, 512})
+        if (r <= rows && entries / r >= kWindowsWanted) return r;
+    return 256;
+}
+// The smallest bucket of the sorted kernel.  It pays where the products bind: FP64 at two and
+// more vectors or complex (64 spinors, M = 500k, 5 to 64 members: 2.15 ms aligned, 1.41 ms
+// sorted; 40 orbitals, two vectors: 0.83, 0.74; 30 orbitals at M = 500k, four vectors, whole
+// kernel: 2.84, 2.60).  One FP64 vector is bound by the table gathers too, and the sort
+// scatters a bucket's rows over warps: 33 to 64 members gain on the 60k space (206 -> 165 us)
+// and lose little on the 2M one (2.78 -> 2.85 ms), smaller ones lose (2M: 3.48 ms from 5 on).
+// The paired-FP32 sums (27 orbitals, one vector: 216 us aligned, 279 sorted; FP32 storage at
+// 4 vectors and fewer) keep the aligned walk.  FP32 storage at 8 vectors, bound by
+// instruction issue, sorts all buckets (30 orbitals, M = 500k: 2.48 ms aligned, 2.37 sorted,
+// 2.44 with the register kernel's eight lanes per small bucket).
+// A pair table of kSmallTable bytes or less stays close to the SMs, and one FP64 vector then
+// sorts from 5 members on too (full CI of 10 orbitals: 162 -> 131 us).
+constexpr int64_t kSmallTable = 1 << 20;
+template <class P, int NV> constexpr int sort_from(bool small_table)
+{
+    if (f32_wide<P, NV>()) return 2;
+    if (!P::kFp64) return kSortBucket + 1;
+    return NV == 1 && sizeof(typename P::SC) == sizeof(double) && !small_table ? 33 : kSmallBucket + 1;
+}
+// The tiled walk takes 32 columns at a time as a mask of doubles for complex FP64 (64
+// spinors, M = 500k: 1.43 -> 1.25 ms) and one FP64 vector (70 orbitals, M = 120k: doubles
+// 1.25 -> 1.02 ms); otherwise in aligned groups (40 orbitals, two vectors: 1.22 ms, 1.29 by
+// mask).
+template <class P, int NV> __host__ __device__ constexpr bool mask_walk()
+{
+    return P::kFp64 && (NV == 1 || sizeof(typename P::SC) == sizeof(zdbl));
+}
+
+// where a launch over the vectors [v0, v0 + NV) finds coefficient v0 + v of determinant I: in
+// C itself ([M][nvec]), or in the split copy of the vector group ([M][NV])
+template <class P, int NV> __device__ __forceinline__ int64_t coef(int64_t I, int nvec, int v0, int v)
+{
+    return P::kSplit ? I * NV + v : I * nvec + v0 + v;
+}
+
+// ------------------------------------------------------------------ walking a row's doubles
+// The doubles of a row among `n` <= 32 consecutive staged members, as a bit mask: bit u is
+// set when member u shares no extra orbital with the row (rc: row_code of the row; code:
+// the members' col_code words).  The row itself and its single excitations leave a 0.
+__device__ __forceinline__ uint32_t doubles_mask(uint32_t rc, const uint32_t *code, int n)
+{
+    uint32_t m = 0;
+    int u = 0;
+    for (; u + 4 <= n; u += 4) {
+        uint32_t g = 0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) g |= (uint32_t)disjoint(rc, code[u + k]) << k;
+        m |= g << u;
+    }
+    for (; u < n; u++) m |= (uint32_t)disjoint(rc, code[u]) << u;
+    return m;
+}
+
+// acc += sum over the set bits u of m of H(row, u) c_u: the pair-table loads of four members
+// are issued before their products, and a member that is no double costs nothing.
+template <class P, int NV>
+__device__ __forceinline__ void walk_mask(uint32_t m, const typename P::TT *__restrict__ trow, const uint32_t *col,
+                                          const typename P::SC *c, typename P::ACC (&acc)[NV])
+{
+    int n = __popc(m);
+    for (; n >= kUnroll; n -= kUnroll) {
+        int j[kUnroll];
+        typename P::TT t[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; u++) {
+            j[u] = __ffs((int)m) - 1;
+            m &= m - 1;
+            t[u] = P::table(trow + col[j[u]]);
+        }
+#pragma unroll
+        for (int u = 0; u < kUnroll; u++)
+#pragma unroll
+            for (int v = 0; v < NV; v++) P::mul_add(acc[v], t[u], c[j[u] * NV + v]);
+#pragma unroll
+        for (int v = 0; v < NV; v++) P::renorm(acc[v]);
+    }
+    // one to three members left
+    const bool two = n & 2, one = n & 1;
+    int j0 = 0, j1 = 0, j2 = 0;
+    typename P::TT t0{}, t1{}, t2{};
+    if (two) {
+        j0 = __ffs((int)m) - 1;
+        m &= m - 1;
+        j1 = __ffs((int)m) - 1;
+        m &= m - 1;
+        t0 = P::table(trow + col[j0]);
+        t1 = P::table(trow + col[j1]);
+    }
+    if (one) {
+        j2 = __ffs((int)m) - 1;
+        t2 = P::table(trow + col[j2]);
+    }
+    if (two) {
+#pragma unroll
+        for (int v = 0; v < NV; v++) {
+            P::mul_add(acc[v], t0, c[j0 * NV + v]);
+            P::mul_add(acc[v], t1, c[j1 * NV + v]);
+        }
+    }
+    if (one) {
+#pragma unroll
+        for (int v = 0; v < NV; v++) P::mul_add(acc[v], t2, c[j2 * NV + v]);
+    }
+#pragma unroll
+    for (int v = 0; v < NV; v++) P::renorm(acc[v]);
+}
+
+// ------------------------------------------------------------------ doubles, small buckets
+// Buckets of at most kSortBucket members.  A CTA owns the whole buckets that start in its
+// kSortRows table rows, and works in three phases:
+//   1. stage the members' codes, determinants and table columns;
+//   2. each thread finds the doubles of its rows as a 64-bit mask over the bucket, gathers
+//      the coefficients of the members that have any, and the CTA sorts the rows by their
+//      number of doubles (a stable counting sort: neighbouring rows of a bucket stay
+//      neighbours and share table sectors).  Rows without a double (27% of the entries of
+//      the 2M-determinant 30-orbital space) end here;
+//   3. each thread walks the set bits of a row's mask.  The rows of a warp have (nearly)
+//      the same count, so its lanes stay on useful products: 97% of the FP64 lane slots
+//      against 65% when lanes walk all members of their buckets.
+constexpr int kSortRows = 448;
+constexpr int kSortCap = kSortRows + kSortBucket;   // rows of a window, at most
+constexpr int kSortRounds = kSortCap / kThreads;    // rows per thread in phases 1 and 2
+static_assert(kSortCap % kThreads == 0, "phase 2 gives every thread the same number of rows");
+
+template <class P, int NV> constexpr size_t sort_smem()
+{
+    return (size_t)kSortCap * (NV * sizeof(typename P::SC) + sizeof(uint2) + 4 * sizeof(uint32_t));
+}
+
+template <class P, int NV, bool RANGED, bool STORE>
+__global__ void __launch_bounds__(kThreads, (min_ctas<P, NV>()))
+k_doubles_sorted(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict__ e_code,
+                 const uint32_t *__restrict__ e_pos, int64_t E, sci::TabRule tr,
+                 const typename P::TT *__restrict__ tab, const typename P::CI *__restrict__ C, int nvec, int v0, typename P::TO *__restrict__ Sout, sci::RowRange rr,
+                 const uint32_t *__restrict__ slot)
+{
+    using SC = typename P::SC;
+    constexpr int kWarps = kThreads / 32;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint16_t s_hist[kWarps][64];
+    __shared__ int s_base[64], s_total;
+    if (chain_last_cta()) return;
+    int64_t r0, r1;
+    window(e_pos, E, kSortRows, r0, r1);
+    if (r0 >= r1) return;
+    const int W = (int)(r1 - r0);
+    SC *s_c = reinterpret_cast<SC *>(smem);
+    uint2 *s_mask = reinterpret_cast<uint2 *>(s_c + kSortCap * NV);
+    uint32_t *s_code = reinterpret_cast<uint32_t *>(s_mask + kSortCap);
+    uint32_t *s_col = s_code + kSortCap;
+    uint32_t *s_idx = s_col + kSortCap;    // determinant, and the member's parity in bit 31
+    uint32_t *s_row = s_idx + kSortCap;    // sorted rows: window row | start of its bucket << 16
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // warp w holds the rows [w * per, (w + 1) * per), 32 at a time
+    const int per = ((W + kWarps - 1) / kWarps + 31) & ~31;
+
+    uint32_t pos[kSortRounds];
+#pragma unroll
+    for (int k = 0; k < kSortRounds; k++) {
+        const int q = wid * per + 32 * k + lane;
+        pos[k] = 0;
+        if (32 * k < per && q < W) {
+            const uint32_t code = e_code[r0 + q];
+            pos[k] = e_pos[r0 + q];
+            uint32_t rowoff, colbase;
+            sci::pair_offsets(tr, sci::code_x(code), sci::code_y(code), rowoff, colbase);
+            s_code[q] = col_code(code);
+            s_col[q] = colbase;
+            s_idx[q] = e_idx[r0 + q] | (uint32_t)sci::code_par(code) << 31;
+        }
+    }
+    for (int t = threadIdx.x; t < kWarps * 64; t += kThreads) (&s_hist[0][0])[t] = 0;
+    __syncthreads();
+
+    int key[kSortRounds], rank[kSortRounds];
+#pragma unroll
+    for (int k = 0; k < kSortRounds; k++) {
+        const int q = wid * per + 32 * k + lane;
+        key[k] = -1;
+        rank[k] = 0;
+        if (pos[k] != 0) {
+            const int size = sci::pos_size(pos[k]), bs = q - sci::pos_off(pos[k]);
+            const uint32_t cc = s_code[q];
+            const uint32_t rc = __byte_perm(cc, 0, 0x1010);   // (x, y, x, y) of the row
+            uint2 m = make_uint2(doubles_mask(rc, s_code + bs, min(size, 32)), 0u);
+            if (size > 32) m.y = doubles_mask(rc, s_code + bs + 32, size - 32);
+            s_mask[q] = m;
+            const int deg = __popc(m.x) + __popc(m.y);
+            const uint32_t ip = s_idx[q];
+            const int64_t I = ip & 0x7fffffffu;
+            if (deg) {
+#pragma unroll
+                for (int v = 0; v < NV; v++) s_c[q * NV + v] = flip(ip >> 31, P::load(C, coef<P, NV>(I, nvec, v0, v)));
+                if (!RANGED || (I >= rr.rb && I < rr.re)) key[k] = 63 - deg;
+            } else if constexpr (STORE) {   // the slot of a row without doubles holds a zero
+#pragma unroll
+                for (int v = 0; v < NV; v++) Sout[(int64_t)slot[r0 + q] * nvec + v0 + v] = typename P::TO{};
+            }
+        }
+        const unsigned act = __ballot_sync(0xffffffffu, key[k] >= 0);
+        unsigned same = 0;
+        if (key[k] >= 0) {
+            same = __match_any_sync(act, key[k]);
+            rank[k] = s_hist[wid][key[k]] + __popc(same & ((1u << lane) - 1u));
+        }
+        __syncwarp();
+        if (key[k] >= 0 && (same >> lane) == 1u) s_hist[wid][key[k]] = (uint16_t)(rank[k] + 1);   // last of its bin
+        __syncwarp();
+    }
+    __syncthreads();
+    if (wid == 0) {   // exclusive prefix over (bin, warp); lane l owns bins 2l and 2l + 1
+        int tot[2];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            int run = 0;
+#pragma unroll
+            for (int w = 0; w < kWarps; w++) {
+                const int c = s_hist[w][2 * lane + h];
+                s_hist[w][2 * lane + h] = (uint16_t)run;
+                run += c;
+            }
+            tot[h] = run;
+        }
+        int inc = tot[0] + tot[1];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += v;
+        }
+        s_base[2 * lane] = inc - tot[0] - tot[1];
+        s_base[2 * lane + 1] = inc - tot[1];
+        if (lane == 31) s_total = inc;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kSortRounds; k++)
+        if (key[k] >= 0) {
+            const int q = wid * per + 32 * k + lane;
+            s_row[s_base[key[k]] + s_hist[wid][key[k]] + rank[k]] =
+                (uint32_t)q | (uint32_t)(q - sci::pos_off(pos[k])) << 16;
+        }
+    __syncthreads();
+
+    const int nrows = s_total;
+    for (int t = threadIdx.x; t < nrows; t += kThreads) {
+        const uint32_t row = s_row[t];
+        const int q = (int)(row & 0xFFFFu), bs = (int)(row >> 16);
+        const uint32_t cc = s_code[q];
+        uint32_t rowoff, colbase;
+        sci::pair_offsets(tr, (int)(cc & 0xFFu), (int)((cc >> 8) & 0xFFu), rowoff, colbase);
+        const typename P::TT *trow = tab + rowoff;
+        const uint2 m = s_mask[q];
+        typename P::ACC acc[NV];
+#pragma unroll
+        for (int v = 0; v < NV; v++) P::clear(acc[v]);
+        walk_mask<P, NV>(m.x, trow, s_col + bs, s_c + bs * NV, acc);
+        if (m.y) walk_mask<P, NV>(m.y, trow, s_col + bs + 32, s_c + (bs + 32) * NV, acc);
+        const uint32_t ip = s_idx[q];
+        const bool par = ip >> 31;
+        if constexpr (STORE) {
+#pragma unroll
+            for (int v = 0; v < NV; v++) Sout[(int64_t)slot[r0 + q] * nvec + v0 + v] = flip(par, P::value(acc[v]));
+        } else {
+#pragma unroll
+            for (int v = 0; v < NV; v++)
+                P::add_out(Sout + (int64_t)(ip & 0x7fffffffu) * nvec + v0 + v, flip(par, P::value(acc[v])));
+        }
+    }
+}
+
+// ------------------------------------------------------------------ doubles, smallest buckets
+// Buckets of S <= kSmallBucket members, which are most of the entries of a selected space
+// (62% of the 2M-determinant 30-orbital space) but few of its pairs (7%).  NV lanes take a
+// bucket, one vector each, with the members in registers: no staging, no barrier, and the
+// members without a double read no coefficient and add nothing.  Lanes of one bucket read the
+// same table entries and neighbouring coefficients.  The L1's rate of scattered 8-byte accesses
+// bounds it (2M space: 145M entries in 0.79 ms); two or four buckets in flight per thread were
+// slower (0.88 ms).
+template <class P, int S, int NV, bool RANGED, bool STORE>
+__global__ void __launch_bounds__(kThreads)
+k_doubles_small(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict__ e_code, int64_t nbuckets,
+                sci::TabRule tr, const typename P::TT *__restrict__ tab, const typename P::CI *__restrict__ C,
+                int nvec, int v0, typename P::TO *__restrict__ Sout, sci::RowRange rr,
+                const uint32_t *__restrict__ slot)
+{
+    if (chain_last_cta()) return;
+    const int64_t t = blockIdx.x * (int64_t)kThreads + threadIdx.x;
+    const int v = (int)(t % NV);
+    const int64_t b = t / NV;
+    if (b >= nbuckets) return;
+    const int64_t g = b * S;
+    uint32_t code[S];
+#pragma unroll
+    for (int i = 0; i < S; i++) code[i] = e_code[g + i];
+    unsigned d[S];   // bit j of d[i]: members i and j are doubles of each other
+#pragma unroll
+    for (int i = 0; i < S; i++) d[i] = 0;
+#pragma unroll
+    for (int i = 0; i < S; i++)
+#pragma unroll
+        for (int j = i + 1; j < S; j++)
+            if (disjoint(row_code(code[i]), col_code(code[j]))) d[i] |= 1u << j, d[j] |= 1u << i;
+    unsigned any = 0;
+#pragma unroll
+    for (int i = 0; i < S; i++) any |= d[i];
+    if (!STORE && any == 0) return;
+    int64_t idx[S];
+    typename P::SC c[S];
+    uint32_t rowoff[S], colbase[S];
+#pragma unroll
+    for (int i = 0; i < S; i++) {
+        idx[i] = 0;
+        c[i] = typename P::SC{};
+        if (d[i]) {
+            idx[i] = e_idx[g + i];
+            c[i] = flip(sci::code_par(code[i]), P::load(C, coef<P, NV>(idx[i], nvec, v0, v)));
+        }
+        sci::pair_offsets(tr, sci::code_x(code[i]), sci::code_y(code[i]), rowoff[i], colbase[i]);
+    }
+    typename P::TT h[S][S];
+#pragma unroll
+    for (int i = 0; i < S; i++)
+#pragma unroll
+        for (int j = 0; j < S; j++) {
+            h[i][j] = typename P::TT{};
+            if (i != j && (d[i] >> j & 1)) h[i][j] = P::table(tab + rowoff[i] + colbase[j]);
+        }
+#pragma unroll
+    for (int i = 0; i < S; i++) {
+        typename P::ACC acc;
+        P::clear(acc);
+#pragma unroll
+        for (int j = 0; j < S; j++)
+            if (i != j && (d[i] >> j & 1)) P::mul_add(acc, h[i][j], c[j]);
+        P::renorm(acc);
+        const typename P::TO out = flip(sci::code_par(code[i]), P::value(acc));
+        if constexpr (STORE) {
+            Sout[(int64_t)slot[g + i] * nvec + v0 + v] = out;
+        } else if (d[i] && (!RANGED || (idx[i] >= rr.rb && idx[i] < rr.re))) {
+            P::add_out(Sout + idx[i] * nvec + v0 + v, out);
+        }
+    }
+}
+
+// ------------------------------------------------------------------ doubles, aligned walk
+// A CTA stages the whole buckets that start in its CH table rows, and each thread walks the
+// members of its row's bucket in order, kUnroll at a time: lanes of one bucket read the same
+// member and neighbouring table entries at every step.  A group with no double of the row is
+// skipped; in the others a member that is no double adds t = 0.
+template <class P, int NV, bool RANGED, bool STORE, int MINB>
+__global__ void __launch_bounds__(kThreads, MINB)
+k_doubles_aligned(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict__ e_code,
+                  const uint32_t *__restrict__ e_pos, int64_t E, int CH, sci::TabRule tr,
+                  const typename P::TT *__restrict__ tab, const typename P::CI *__restrict__ C, int nvec, int v0, typename P::TO *__restrict__ Sout, sci::RowRange rr,
+                  const uint32_t *__restrict__ slot)
+{
+    using SC = typename P::SC;
+    using TT = typename P::TT;
+    extern __shared__ __align__(16) unsigned char smem[];
+    if (chain_last_cta()) return;
+    int64_t r0, r1;
+    window(e_pos, E, CH, r0, r1);
+    if (r0 >= r1) return;
+    const int W = (int)(r1 - r0);
+    SC *s_c = reinterpret_cast<SC *>(smem);
+    const size_t cbytes = ((size_t)W * NV * sizeof(SC) + 15) & ~(size_t)15;
+    uint2 *s_kc = reinterpret_cast<uint2 *>(smem + cbytes);
+    uint16_t *s_own = reinterpret_cast<uint16_t *>(smem + cbytes + (size_t)W * sizeof(uint2));
+    int nrows = W;
+    if constexpr (RANGED) {
+        nrows = owned_rows(e_idx, r0, W, rr, s_own);
+        if (nrows == 0) return;
+    }
+    for (int q = threadIdx.x; q < W; q += blockDim.x) {
+        const int64_t g = r0 + q;
+        const uint32_t idx = e_idx[g], code = e_code[g];
+        uint32_t rowoff, colbase;
+        sci::pair_offsets(tr, sci::code_x(code), sci::code_y(code), rowoff, colbase);
+        s_kc[q] = make_uint2(col_code(code), colbase);
+        const bool par = sci::code_par(code);
+#pragma unroll
+        for (int v = 0; v < NV; v++) s_c[q * NV + v] = flip(par, P::load(C, coef<P, NV>(idx, nvec, v0, v)));
+    }
+    __syncthreads();
+    for (int t_ = threadIdx.x; t_ < nrows; t_ += blockDim.x) {
+        const int q0 = RANGED ? (int)s_own[t_] : t_;
+        const uint32_t code = e_code[r0 + q0], pos = e_pos[r0 + q0];
+        uint32_t rowoff, colbase;
+        sci::pair_offsets(tr, sci::code_x(code), sci::code_y(code), rowoff, colbase);
+        // FP64 policies walk the members other than the row itself, j standing for bucket
+        // position j + (j >= q0); the paired-FP32 ones all members (see the policies)
+        const int bs = q0 - sci::pos_off(pos), je = bs + sci::pos_size(pos) - (P::kSkipSelf ? 1 : 0);
+        auto member = [&](int j) { return P::kSkipSelf ? j + (j >= q0) : j; };
+        const uint32_t rc = row_code(code);
+        const TT *trow = tab + rowoff;
+        typename P::ACC acc[NV];
+#pragma unroll
+        for (int v = 0; v < NV; v++) P::clear(acc[v]);
+        int j = bs;
+        for (; j + kUnroll <= je; j += kUnroll) {
+            uint2 kc[kUnroll];
+            TT t[kUnroll];
+            unsigned vm = 0;
+#pragma unroll
+            for (int u = 0; u < kUnroll; u++) {
+                kc[u] = s_kc[member(j + u)];
+                vm |= (unsigned)disjoint(rc, kc[u].x) << u;
+            }
+            if (vm == 0) continue;
+#pragma unroll
+            for (int u = 0; u < kUnroll; u++) {
+                t[u] = TT{};
+                if (vm & (1u << u)) t[u] = P::table(trow + kc[u].y);
+            }
+#pragma unroll
+            for (int u = 0; u < kUnroll; u++)
+#pragma unroll
+                for (int v = 0; v < NV; v++) P::mul_add(acc[v], t[u], s_c[member(j + u) * NV + v]);
+#pragma unroll
+            for (int v = 0; v < NV; v++) P::renorm(acc[v]);
+        }
+        for (; j < je; j++) {
+            const int m = member(j);
+            const uint2 kc = s_kc[m];
+            if (!disjoint(rc, kc.x)) continue;
+            const TT t = P::table(trow + kc.y);
+#pragma unroll
+            for (int v = 0; v < NV; v++) P::mul_add(acc[v], t, s_c[m * NV + v]);
+        }
+        const bool par = sci::code_par(code);
+        if constexpr (STORE) {
+#pragma unroll
+            for (int v = 0; v < NV; v++) Sout[(int64_t)slot[r0 + q0] * nvec + v0 + v] = flip(par, P::value(acc[v]));
+        } else {
+            const uint32_t idx = e_idx[r0 + q0];
+#pragma unroll
+            for (int v = 0; v < NV; v++) P::add_out(Sout + (int64_t)idx * nvec + v0 + v, flip(par, P::value(acc[v])));
+        }
+    }
+}
+
+// ------------------------------------------------------------------ doubles, tiled
+// (N-2) buckets of more than tile_b members (sci_set_tile_threshold) are too large to
+// stage whole beside a window, so they run here.  A CTA takes kTileRows consecutive
+// members of one bucket as its rows (one per thread) and streams the bucket's members
+// through shared memory in column tiles, each staged once per CTA; every thread walks a
+// column tile against its row as the window kernels walk a bucket (disjointness test, one
+// table load per double, the FMAs), so a row sums the same products.  The row itself and
+// its single excitations fail the disjointness test and add nothing.  All threads of a
+// CTA share the bucket, so trip counts are uniform and the barriers are CTA-wide.
 // shared memory of the tiled kernel: at most this, which needs no opt-in
 constexpr size_t kTiledSmem = 48 * 1024;
 
-// C holds coefficient v of determinant I at C[I * cstride + coff + v].  With few tiles
+// C holds coefficient v of determinant I at C[coef<P, NV>(I, nvec, v0, v)].  With few tiles
 // (a handful of very large buckets) the columns of a bucket are also split: CTA row y of
 // the grid (gridDim.y = nsplit) takes the y-th of nsplit equal runs of column tiles and
 // adds its partial row sums atomically (nsplit = 1 in the deterministic mode, where one
@@ -688,17 +863,21 @@ __global__ void __launch_bounds__(kThreads)
 k_doubles_tiled(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict__ e_code,
                 const uint32_t *__restrict__ e_pos, const uint32_t *__restrict__ tiles, int64_t ntiles, int TCOL,
                 sci::TabRule tr, const typename P::TT *__restrict__ tab, const typename P::CI *__restrict__ C,
-                int cstride, int coff, int nvec, int v0, typename P::TO *__restrict__ Sout, sci::RowRange rr,
+                int nvec, int v0, typename P::TO *__restrict__ Sout, sci::RowRange rr,
                 const uint32_t *__restrict__ slot)
 {
+    if (chain_last_cta()) return;
     const int nsplit = STORE ? 1 : (int)gridDim.y;
     using SC = typename P::SC;
     using TT = typename P::TT;
     using ACC = typename P::ACC;
     extern __shared__ __align__(16) unsigned char smem[];
     SC *s_c = reinterpret_cast<SC *>(smem);
-    uint2 *s_kc = reinterpret_cast<uint2 *>(smem + (((size_t)TCOL * NV * sizeof(SC) + 15) & ~(size_t)15));
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    // codes and columns, apart for the walk by masks and as pairs for the aligned one
+    uint32_t *s_code = reinterpret_cast<uint32_t *>(smem + (((size_t)TCOL * NV * sizeof(SC) + 15) & ~(size_t)15));
+    uint32_t *s_col = s_code + TCOL;
+    uint2 *s_kc = reinterpret_cast<uint2 *>(s_code);
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x - 1) {
         const int64_t r0 = tiles[t];
         const uint32_t pos0 = e_pos[r0];
         const int64_t bs = r0 - sci::pos_off(pos0);
@@ -736,45 +915,55 @@ k_doubles_tiled(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict__
                 const uint32_t idx = e_idx[g], code = e_code[g];
                 uint32_t rowoff, colbase;
                 sci::pair_offsets(tr, sci::code_x(code), sci::code_y(code), rowoff, colbase);
-                s_kc[q] = make_uint2(col_code(code), colbase);
+                if constexpr (mask_walk<P, NV>()) {
+                    s_code[q] = col_code(code);
+                    s_col[q] = colbase;
+                } else {
+                    s_kc[q] = make_uint2(col_code(code), colbase);
+                }
                 const bool pq = sci::code_par(code);
 #pragma unroll
-                for (int v = 0; v < NV; v++) s_c[q * NV + v] = flip(pq, P::load(C, (int64_t)idx * cstride + coff + v));
+                for (int v = 0; v < NV; v++) s_c[q * NV + v] = flip(pq, P::load(C, coef<P, NV>(idx, nvec, v0, v)));
             }
             __syncthreads();
             if (!active) continue;
-            int j = 0;
-            for (; j + kUnroll <= n; j += kUnroll) {
-                uint2 kc[kUnroll];
-                TT tv[kUnroll];
-                unsigned vm = 0;
+            if constexpr (mask_walk<P, NV>()) {
+                for (int j = 0; j < n; j += 32)
+                    walk_mask<P, NV>(doubles_mask(rc, s_code + j, min(32, n - j)), trow, s_col + j, s_c + j * NV, acc);
+            } else {
+                int j = 0;
+                for (; j + kUnroll <= n; j += kUnroll) {
+                    uint2 kc[kUnroll];
+                    TT tv[kUnroll];
+                    unsigned vm = 0;
 #pragma unroll
-                for (int u = 0; u < kUnroll; u++) {
-                    kc[u] = s_kc[j + u];
-                    vm |= (unsigned)disjoint(rc, kc[u].x) << u;
+                    for (int u = 0; u < kUnroll; u++) {
+                        kc[u] = s_kc[j + u];
+                        vm |= (unsigned)disjoint(rc, kc[u].x) << u;
+                    }
+                    if (vm == 0) continue;
+#pragma unroll
+                    for (int u = 0; u < kUnroll; u++) {
+                        tv[u] = TT{};
+                        if (vm & (1u << u)) tv[u] = P::table(trow + kc[u].y);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kUnroll; u++)
+#pragma unroll
+                        for (int v = 0; v < NV; v++) P::mul_add(acc[v], tv[u], s_c[(j + u) * NV + v]);
+#pragma unroll
+                    for (int v = 0; v < NV; v++) P::renorm(acc[v]);
                 }
-                if (vm == 0) continue;
+                for (; j < n; j++) {
+                    const uint2 kc = s_kc[j];
+                    if (!disjoint(rc, kc.x)) continue;
+                    const TT tv = P::table(trow + kc.y);
 #pragma unroll
-                for (int u = 0; u < kUnroll; u++) {
-                    tv[u] = TT{};
-                    if (vm & (1u << u)) tv[u] = P::table(trow + kc[u].y);
+                    for (int v = 0; v < NV; v++) P::mul_add(acc[v], tv, s_c[j * NV + v]);
                 }
-#pragma unroll
-                for (int u = 0; u < kUnroll; u++)
-#pragma unroll
-                    for (int v = 0; v < NV; v++) P::mul_add(acc[v], tv[u], s_c[(j + u) * NV + v]);
 #pragma unroll
                 for (int v = 0; v < NV; v++) P::renorm(acc[v]);
             }
-            for (; j < n; j++) {
-                const uint2 kc = s_kc[j];
-                if (!disjoint(rc, kc.x)) continue;
-                const TT tv = P::table(trow + kc.y);
-#pragma unroll
-                for (int v = 0; v < NV; v++) P::mul_add(acc[v], tv, s_c[j * NV + v]);
-            }
-#pragma unroll
-            for (int v = 0; v < NV; v++) P::renorm(acc[v]);
         }
         if (active) {
             if constexpr (STORE) {
@@ -797,6 +986,7 @@ k_singles(const uint32_t *__restrict__ e_idx, const uint64_t *__restrict__ e_S, 
           const TC *__restrict__ C, int nvec, int v0, typename AccOf<TS>::type *__restrict__ Sout, sci::RowRange rr, const uint32_t *__restrict__ slot)
 {
     using TA = typename AccOf<TS>::type;
+    chain_next();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < E; p += (int64_t)gridDim.x * blockDim.x) {
         if constexpr (RANGED) {
             const int64_t I = e_idx[p];
@@ -849,6 +1039,7 @@ k_singles(const uint32_t *__restrict__ e_idx, const uint64_t *__restrict__ e_S, 
             for (int v = 0; v < NV; v++) red_add(Sout + (int64_t)idx * nvec + v0 + v, flip(par, acc[v]));
         }
     }
+    chain_wait();
 }
 
 // ------------------------------------------------------------------ singles, paired FP32
@@ -1057,52 +1248,113 @@ Tabs tabs_of(const sci_ctx *ctx)
 // the tiled kernel over the buckets of [0, sp.big) (nothing when there are none)
 template <class P, bool RG, bool ST, int NV>
 int launch_tiled(sci_ctx *ctx, const Tabs &T, const sci::Split &sp, const typename P::TT *tab,
-                 const typename P::CI *C, int cstride, int coff, int nvec, int v0, typename P::TO *S)
+                 const typename P::CI *C, int nvec, int v0, typename P::TO *S, bool &chained)
 {
     if (sp.ntiles == 0) return SCI_OK;
     const size_t per = NV * sizeof(typename P::SC) + sizeof(uint2);
     int tcol = (int)std::min<size_t>(1024, (kTiledSmem - 16) / per) & ~31;
-    const size_t smem = (((size_t)tcol * NV * sizeof(typename P::SC) + 15) & ~(size_t)15) + (size_t)tcol * sizeof(uint2);
-    const int64_t grid = std::min<int64_t>(sp.ntiles, 152 * 16);
-    // few tiles: split the columns too, up to the column tiles of the largest bucket, for
-    // about 8 CTAs per SM (not in the deterministic mode, whose slots have one writer)
+    // with few tiles the columns are split too, in runs of 64 members and more, for four
+    // waves of CTAs: tiles of unequal buckets leave the last wave nearly empty otherwise (not
+    // in the deterministic mode, whose slots have one writer).  70 orbitals, M = 120k: 942 us
+    // at one wave, 823 at four; 45 spinors, M = 118k, two paired-FP32 vectors: 234 tiles, 181
+    // us unsplit, 121.  Wide vector groups pay for each split with as many atomics per row
+    // and stop at one wave (56 orbitals, 8 vectors: 6.43 ms at one, 6.84 at four).
     int nsplit = 1;
-    if (!ST && sp.ntiles < 152 * 8) {
-        const int64_t want = (152 * 8 + sp.ntiles - 1) / sp.ntiles;
-        const int64_t most = (ctx->maxb2 + tcol - 1) / tcol;
-        nsplit = (int)std::max<int64_t>(1, std::min<int64_t>({want, most, 65535}));
+    const int64_t ctas = 152 * (NV * sizeof(typename P::SC) >= sci::kWideRowBytes ? 8 : 32);
+    if (!ST && sp.ntiles < ctas) {
+        const int64_t want = (ctas + sp.ntiles - 1) / sp.ntiles;
+        const int cols = (int)std::max<int64_t>(64, ((ctx->maxb2 + want - 1) / want + 31) & ~(int64_t)31);
+        tcol = std::min(tcol, cols);
+        nsplit = (int)std::min<int64_t>({want, (ctx->maxb2 + tcol - 1) / tcol, 65535});
     }
-    k_doubles_tiled<P, NV, RG, ST><<<dim3((unsigned)grid, (unsigned)nsplit), kThreads, smem, ctx->stream>>>(
-        T.e2_idx, T.e2_code, T.e2_pos, T.tiles(), sp.ntiles, tcol, tab_rule(ctx), tab, C, cstride, coff, nvec, v0, S,
-        T.rr, ST ? ctx->det_inv2 : nullptr);
-    return sci_cuda_check(ctx, cudaGetLastError(), "k_doubles_tiled launch");
+    const size_t smem = (((size_t)tcol * NV * sizeof(typename P::SC) + 15) & ~(size_t)15) + (size_t)tcol * sizeof(uint2);
+    cudaError_t e = launch_chained(chained, k_doubles_tiled<P, NV, RG, ST>,
+                                   dim3((unsigned)sp.ntiles + 1, (unsigned)nsplit), smem, ctx->stream, T.e2_idx,
+                                   T.e2_code, T.e2_pos, T.tiles(), sp.ntiles, tcol, tab_rule(ctx), tab, C, nvec, v0, S,
+                                   T.rr, ST ? ctx->det_inv2 : nullptr);
+    chained = true;
+    return sci_cuda_check(ctx, e, "k_doubles_tiled launch");
 }
 
 // staged bytes per window row: NV coefficients, the (code, offset) pair, and in a RANGED
 // launch the row's slot in the owned-row list
 template <bool RG> constexpr size_t row_extra() { return RG ? 8 + sizeof(uint16_t) : 8; }
 
-template <bool RG, bool ST, typename TS, typename TC, int NV>
-int launch_doubles(sci_ctx *ctx, const Tabs &T, const TS *tab, const TC *C, typename AccOf<TS>::type *S, int nvec,
-                   int v0)
+// the doubles of one vector group, by bucket size: the tiled kernel above the tile threshold,
+// the aligned walk down to kSortBucket members, then the sorted kernel, the aligned walk
+// and the register kernel as sort_from() and kSmallBucket say
+template <class P, bool RG, bool ST, int NV>
+int launch_doubles(sci_ctx *ctx, const Tabs &T, const typename P::TT *tab, const typename P::CI *C, int nvec, int v0,
+                   typename P::TO *S, bool &chained)
 {
     if (T.e2 == 0) return SCI_OK;
-    const size_t per = NV * sizeof(TS) + row_extra<RG>();
+    const size_t per = NV * sizeof(typename P::SC) + row_extra<RG>();
     const sci::Split &sp = T.split(per);
-    int rc = launch_tiled<PolF64<TS, TC>, RG, ST, NV>(ctx, T, sp, tab, C, nvec, v0, nvec, v0, S);
-    const int64_t b = sp.big, E = T.e2 - b;
-    if (rc != SCI_OK || E == 0) return rc;
-    size_t smem = 0;
-    int ch = choose_rows(sp.maxb_small, per, smem);
-    if (ch < 0) return sci_fail(ctx, SCI_ERR_OVERFLOW, "bucket too large for shared memory");
-    auto kern = k_doubles<TS, TC, NV, RG, ST>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return sci_cuda_check(ctx, e, "cudaFuncSetAttribute");
-    int64_t blocks = (E + ch - 1) / ch;
-    kern<<<(unsigned)blocks, kThreads, smem, ctx->stream>>>(T.e2_idx + b, T.e2_code + b, T.e2_pos + b, E, ch,
-                                                          tab_rule(ctx), tab, C, nvec, v0, S, T.rr,
-                                                          ST ? ctx->det_inv2 + b : nullptr);
-    return sci_cuda_check(ctx, cudaGetLastError(), "k_doubles launch");
+    int rc = launch_tiled<P, RG, ST, NV>(ctx, T, sp, tab, C, nvec, v0, S, chained);
+    // the entries from lo on of buckets of at most `maxb` members, up to hi
+    auto aligned = [&](auto kern, int64_t lo, int64_t hi, int maxb, int rows) -> int {
+        if (hi <= lo) return SCI_OK;
+        size_t smem = 0;
+        const int ch = choose_rows(maxb, per, smem, rows);
+        if (ch < 0) return sci_fail(ctx, SCI_ERR_OVERFLOW, "bucket too large for shared memory");
+        if (smem > 48 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return sci_cuda_check(ctx, e, "cudaFuncSetAttribute");
+        }
+        cudaError_t e = launch_chained(chained, kern, dim3((unsigned)((hi - lo + ch - 1) / ch) + 1), smem, ctx->stream,
+                                       T.e2_idx + lo, T.e2_code + lo, T.e2_pos + lo, hi - lo, ch, tab_rule(ctx), tab,
+                                       C, nvec, v0, S, T.rr, ST ? ctx->det_inv2 + lo : nullptr);
+        chained = true;
+        return sci_cuda_check(ctx, e, "k_doubles_aligned launch");
+    };
+    constexpr int rows = f32_wide<P, NV>() ? SCI_F32_ROWS : kRowsPerCta;
+    // the first entry of each part: the tiles end at b, the middle buckets at m, the sorted
+    // ones at so, the aligned ones of five members and more at sm
+    const int64_t *above = T.ts->above;
+    const int64_t b = sp.big, m = std::max(b, above[kSortBucket]);
+    constexpr int lowest = sort_from<P, NV>(true);
+    const int from = sort_from<P, NV>(ctx->tab_elems * (int64_t)sizeof(typename P::TT) <= kSmallTable);
+    const int64_t sm = lowest <= kSmallBucket ? T.e2 : std::max(m, above[kSmallBucket]);
+    const int64_t so = from > kSortBucket ? m : std::min(sm, std::max(m, above[from - 1]));
+    if (rc == SCI_OK)
+        rc = aligned(k_doubles_aligned<P, NV, RG, ST, wide_ctas<P, NV>()>, b, m, sp.maxb_small,
+                     window_rows(m - b, rows));
+    if (rc != SCI_OK) return rc;
+    if constexpr (lowest <= kSortBucket) {
+        if (so > m) {
+            constexpr size_t smem = sort_smem<P, NV>();
+            auto kern = k_doubles_sorted<P, NV, RG, ST>;
+            if constexpr (smem > 47 * 1024) {   // static shared memory counts against the 48 KB too
+                cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (e != cudaSuccess) return sci_cuda_check(ctx, e, "cudaFuncSetAttribute");
+            }
+            cudaError_t e = launch_chained(chained, kern, dim3((unsigned)((so - m + kSortRows - 1) / kSortRows) + 1),
+                                           smem, ctx->stream, T.e2_idx + m, T.e2_code + m, T.e2_pos + m, so - m,
+                                           tab_rule(ctx), tab, C, nvec, v0, S, T.rr, ST ? ctx->det_inv2 + m : nullptr);
+            chained = true;
+            if ((rc = sci_cuda_check(ctx, e, "k_doubles_sorted launch")) != SCI_OK) return rc;
+        }
+    }
+    if constexpr (lowest > kSmallBucket) {
+        if constexpr (sort_from<P, NV>(false) > kSmallBucket + 1)
+            rc = aligned(k_doubles_aligned<P, NV, RG, ST, min_ctas<P, NV>()>, so, sm, std::min(from - 1, sp.maxb_small),
+                         rows);
+        if (rc != SCI_OK) return rc;
+        auto small = [&](auto kern, int size) -> int {   // the buckets of `size` members
+            const int64_t lo = std::max(m, above[size]), hi = std::max(m, above[size - 1]);
+            if (hi == lo) return SCI_OK;
+            const int64_t nb = (hi - lo) / size;
+            cudaError_t e = launch_chained(chained, kern, dim3((unsigned)((nb * NV + kThreads - 1) / kThreads) + 1), 0,
+                                           ctx->stream, T.e2_idx + lo, T.e2_code + lo, nb, tab_rule(ctx), tab, C, nvec,
+                                           v0, S, T.rr, ST ? ctx->det_inv2 + lo : nullptr);
+            chained = true;
+            return sci_cuda_check(ctx, e, "k_doubles_small launch");
+        };
+        rc = small(k_doubles_small<P, 4, NV, RG, ST>, 4);
+        if (rc == SCI_OK) rc = small(k_doubles_small<P, 3, NV, RG, ST>, 3);
+        if (rc == SCI_OK) rc = small(k_doubles_small<P, 2, NV, RG, ST>, 2);
+    }
+    return rc;
 }
 
 // paired-FP32 doubles: real (float2 table, float2 staged c) or complex (float4 / float4)
@@ -1110,13 +1362,6 @@ template <bool RG, bool ST, bool CPLX, int NV>
 int launch_doubles_ds(sci_ctx *ctx, const Tabs &T, const void *C, void *S, int nvec, int v0)
 {
     if (T.e2 == 0) return SCI_OK;
-    const size_t per = NV * (CPLX ? sizeof(float4) : sizeof(float2)) + row_extra<RG>();
-    const sci::Split &sp = T.split(per);
-    const int64_t b = sp.big, E = T.e2 - b;
-    size_t smem = 0;
-    int ch = E > 0 ? choose_rows(sp.maxb_small, per, smem) : 0;
-    if (ch < 0) return sci_fail(ctx, SCI_ERR_OVERFLOW, "bucket too large for shared memory");
-    cudaError_t e;
     // the vector group, split into paired floats in the context's c_ds buffer
     // (64 bytes per determinant: up to 8 real or 4 complex coefficients)
     if constexpr (CPLX)
@@ -1125,32 +1370,12 @@ int launch_doubles_ds(sci_ctx *ctx, const Tabs &T, const void *C, void *S, int n
     else
         k_split_c<<<grid_for(ctx->M * NV), kThreads, 0, ctx->stream>>>((const double *)C, ctx->M, nvec, v0, NV,
                                                                        (float2 *)ctx->c_ds);
-    int rc;
+    SCI_CK(cudaGetLastError());
+    bool chained = false;   // the first launch reads the split copy made just before
     if constexpr (CPLX)
-        rc = launch_tiled<PolDSZ, RG, ST, NV>(ctx, T, sp, (const float4 *)ctx->tab_ds, (const float4 *)ctx->c_ds, NV,
-                                              0, nvec, v0, (zdbl *)S);
+        return launch_doubles<PolDSZ, RG, ST, NV>(ctx, T, (const float4 *)ctx->tab_ds, (const float4 *)ctx->c_ds, nvec, v0, (zdbl *)S, chained);
     else
-        rc = launch_tiled<PolDS, RG, ST, NV>(ctx, T, sp, (const float2 *)ctx->tab_ds, (const float2 *)ctx->c_ds, NV,
-                                             0, nvec, v0, (double *)S);
-    if (rc != SCI_OK || E == 0) return rc;
-    const int64_t blocks = (E + ch - 1) / ch;
-    const uint32_t *slot = ST ? ctx->det_inv2 + b : nullptr;
-    if constexpr (CPLX) {
-        auto kern = k_doubles_dsz<NV, RG, ST>;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return sci_cuda_check(ctx, e, "cudaFuncSetAttribute");
-        kern<<<(unsigned)blocks, kThreads, smem, ctx->stream>>>(T.e2_idx + b, T.e2_code + b, T.e2_pos + b, E, ch,
-                                                              tab_rule(ctx), (const float4 *)ctx->tab_ds,
-                                                              (const float4 *)ctx->c_ds, nvec, v0, (zdbl *)S, T.rr, slot);
-    } else {
-        auto kern = k_doubles_ds<NV, RG, ST>;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return sci_cuda_check(ctx, e, "cudaFuncSetAttribute");
-        kern<<<(unsigned)blocks, kThreads, smem, ctx->stream>>>(T.e2_idx + b, T.e2_code + b, T.e2_pos + b, E, ch,
-                                                              tab_rule(ctx), (const float2 *)ctx->tab_ds,
-                                                              (const float2 *)ctx->c_ds, nvec, v0, (double *)S, T.rr, slot);
-    }
-    return sci_cuda_check(ctx, cudaGetLastError(), "k_doubles_ds launch");
+        return launch_doubles<PolDS, RG, ST, NV>(ctx, T, (const float2 *)ctx->tab_ds, (const float2 *)ctx->c_ds, nvec, v0, (double *)S, chained);
 }
 
 template <bool RG, bool ST, bool CPLX>
@@ -1165,7 +1390,9 @@ int ds_groups(sci_ctx *ctx, const Tabs &T, const void *C, void *S, int nvec)
         size_t smem_probe = 0;
         while (g > 1 && choose_rows(T.maxb_small(), g * unit + row_extra<RG>(), smem_probe) < 0) g >>= 1;
         switch (g) {
-        case 8: rc = launch_doubles_ds<RG, ST, CPLX, 8>(ctx, T, C, S, nvec, v0); break;
+        case 8:
+            if constexpr (!CPLX) rc = launch_doubles_ds<RG, ST, CPLX, 8>(ctx, T, C, S, nvec, v0);
+            break;
         case 4: rc = launch_doubles_ds<RG, ST, CPLX, 4>(ctx, T, C, S, nvec, v0); break;
         case 2: rc = launch_doubles_ds<RG, ST, CPLX, 2>(ctx, T, C, S, nvec, v0); break;
         default: rc = launch_doubles_ds<RG, ST, CPLX, 1>(ctx, T, C, S, nvec, v0); break;
@@ -1176,42 +1403,21 @@ int ds_groups(sci_ctx *ctx, const Tabs &T, const void *C, void *S, int nvec)
 }
 
 // FP32-storage doubles (SCI_PREC_F32_STORE_F64_ACC)
-template <bool RG, bool ST, int NV>
-int launch_doubles_f32(sci_ctx *ctx, const Tabs &T, const float *C, double *S, int nvec, int v0)
-{
-    if (T.e2 == 0) return SCI_OK;
-    const size_t per = NV * sizeof(float) + row_extra<RG>();
-    const sci::Split &sp = T.split(per);
-    int rc = launch_tiled<PolF32, RG, ST, NV>(ctx, T, sp, ctx->tab32, C, nvec, v0, nvec, v0, S);
-    const int64_t b = sp.big, E = T.e2 - b;
-    if (rc != SCI_OK || E == 0) return rc;
-    size_t smem = 0;
-    int ch = choose_rows(sp.maxb_small, per, smem, NV >= 8 ? SCI_F32_ROWS : kRowsPerCta);
-    if (ch < 0) return sci_fail(ctx, SCI_ERR_OVERFLOW, "bucket too large for shared memory");
-    int64_t blocks = (E + ch - 1) / ch;
-    auto kern = k_doubles_f32<NV, RG, ST>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return sci_cuda_check(ctx, e, "cudaFuncSetAttribute");
-    kern<<<(unsigned)blocks, kThreads, smem, ctx->stream>>>(T.e2_idx + b, T.e2_code + b, T.e2_pos + b, E, ch,
-                                                          tab_rule(ctx), ctx->tab32, C, nvec, v0, S, T.rr,
-                                                          ST ? ctx->det_inv2 + b : nullptr);
-    return sci_cuda_check(ctx, cudaGetLastError(), "k_doubles_f32 launch");
-}
-
 template <bool RG, bool ST>
 int f32_groups(sci_ctx *ctx, const Tabs &T, const float *C, double *S, int nvec)
 {
     int rc = SCI_OK;
+    bool chained = false;
     for (int v0 = 0; v0 < nvec && rc == SCI_OK;) {
         int left = nvec - v0;
         int g = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
         size_t smem_probe = 0;
         while (g > 1 && choose_rows(T.maxb_small(), g * sizeof(float) + row_extra<RG>(), smem_probe) < 0) g >>= 1;
         switch (g) {
-        case 8: rc = launch_doubles_f32<RG, ST, 8>(ctx, T, C, S, nvec, v0); break;
-        case 4: rc = launch_doubles_f32<RG, ST, 4>(ctx, T, C, S, nvec, v0); break;
-        case 2: rc = launch_doubles_f32<RG, ST, 2>(ctx, T, C, S, nvec, v0); break;
-        default: rc = launch_doubles_f32<RG, ST, 1>(ctx, T, C, S, nvec, v0); break;
+        case 8: rc = launch_doubles<PolF32, RG, ST, 8>(ctx, T, ctx->tab32, C, nvec, v0, S, chained); break;
+        case 4: rc = launch_doubles<PolF32, RG, ST, 4>(ctx, T, ctx->tab32, C, nvec, v0, S, chained); break;
+        case 2: rc = launch_doubles<PolF32, RG, ST, 2>(ctx, T, ctx->tab32, C, nvec, v0, S, chained); break;
+        default: rc = launch_doubles<PolF32, RG, ST, 1>(ctx, T, ctx->tab32, C, nvec, v0, S, chained); break;
         }
         v0 += g;
     }
@@ -1261,7 +1467,9 @@ int ds_singles_groups(sci_ctx *ctx, const Tabs &T, const void *C, void *S, int n
         int g = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
         if (CPLX && g > 4) g = 4;
         switch (g) {
-        case 8: rc = launch_singles_ds<RG, ST, CPLX, 8, TC>(ctx, T, C, S, nvec, v0); break;
+        case 8:
+            if constexpr (!CPLX) rc = launch_singles_ds<RG, ST, CPLX, 8, TC>(ctx, T, C, S, nvec, v0);
+            break;
         case 4: rc = launch_singles_ds<RG, ST, CPLX, 4, TC>(ctx, T, C, S, nvec, v0); break;
         case 2: rc = launch_singles_ds<RG, ST, CPLX, 2, TC>(ctx, T, C, S, nvec, v0); break;
         default: rc = launch_singles_ds<RG, ST, CPLX, 1, TC>(ctx, T, C, S, nvec, v0); break;
@@ -1272,21 +1480,23 @@ int ds_singles_groups(sci_ctx *ctx, const Tabs &T, const void *C, void *S, int n
 }
 
 template <bool RG, bool ST, typename TS, typename TC, int NV>
-int launch_singles(sci_ctx *ctx, const Tabs &T, const TC *C, typename AccOf<TS>::type *S, int nvec, int v0)
+int launch_singles(sci_ctx *ctx, const Tabs &T, const TC *C, typename AccOf<TS>::type *S, int nvec, int v0, bool &chained)
 {
     if (T.e1 == 0) return SCI_OK;
     auto kern = ctx->nwords == 4   ? k_singles<TS, TC, NV, RG, ST, 4>
                 : ctx->nwords == 3 ? k_singles<TS, TC, NV, RG, ST, 3>
                 : ctx->nwords == 2 ? k_singles<TS, TC, NV, RG, ST, 2>
                                    : k_singles<TS, TC, NV, RG, ST, 1>;
-    kern<<<grid_for(T.e1), kThreads, 0, ctx->stream>>>(T.e1_idx, T.e1_S, T.e1_meta, T.e1, ctx->norb, ref_words(ctx),
-                                                       (const TS *)ctx->fref, (const TS *)ctx->g_so, C,
-                                                       nvec, v0, S, T.rr, ST ? ctx->det_inv1 : nullptr);
-    return sci_cuda_check(ctx, cudaGetLastError(), "k_singles launch");
+    cudaError_t e = launch_chained(chained, kern, dim3(grid_for(T.e1)), 0, ctx->stream, T.e1_idx, T.e1_S, T.e1_meta,
+                                   T.e1, ctx->norb, ref_words(ctx), (const TS *)ctx->fref, (const TS *)ctx->g_so, C,
+                                   nvec, v0, S, T.rr, ST ? ctx->det_inv1 : nullptr);
+    chained = true;
+    return sci_cuda_check(ctx, e, "k_singles launch");
 }
 
 template <bool RG, bool ST, typename TS, typename TC>
-int sigma_groups(sci_ctx *ctx, const Tabs &T, const TS *tab, const TC *C, typename AccOf<TS>::type *S, int nvec)
+int sigma_groups(sci_ctx *ctx, const Tabs &T, const TS *tab, const TC *C, typename AccOf<TS>::type *S, int nvec,
+                 bool &chained)
 {
     int rc = SCI_OK;
     for (int v0 = 0; v0 < nvec && rc == SCI_OK;) {
@@ -1296,10 +1506,13 @@ int sigma_groups(sci_ctx *ctx, const Tabs &T, const TS *tab, const TC *C, typena
         size_t smem_probe = 0;  // shrink the vector group until its window fits
         while (g > 1 && choose_rows(T.maxb_small(), g * sizeof(TS) + row_extra<RG>(), smem_probe) < 0) g >>= 1;
         switch (g) {
-        case 8: rc = launch_doubles<RG, ST, TS, TC, 8>(ctx, T, tab, C, S, nvec, v0); break;
-        case 4: rc = launch_doubles<RG, ST, TS, TC, 4>(ctx, T, tab, C, S, nvec, v0); break;
-        case 2: rc = launch_doubles<RG, ST, TS, TC, 2>(ctx, T, tab, C, S, nvec, v0); break;
-        default: rc = launch_doubles<RG, ST, TS, TC, 1>(ctx, T, tab, C, S, nvec, v0); break;
+        case 8:
+            if constexpr (sizeof(TS) == sizeof(double))
+                rc = launch_doubles<PolF64<TS, TC>, RG, ST, 8>(ctx, T, tab, C, nvec, v0, S, chained);
+            break;
+        case 4: rc = launch_doubles<PolF64<TS, TC>, RG, ST, 4>(ctx, T, tab, C, nvec, v0, S, chained); break;
+        case 2: rc = launch_doubles<PolF64<TS, TC>, RG, ST, 2>(ctx, T, tab, C, nvec, v0, S, chained); break;
+        default: rc = launch_doubles<PolF64<TS, TC>, RG, ST, 1>(ctx, T, tab, C, nvec, v0, S, chained); break;
         }
         v0 += g;
     }
@@ -1307,16 +1520,16 @@ int sigma_groups(sci_ctx *ctx, const Tabs &T, const TS *tab, const TC *C, typena
 }
 
 template <bool RG, bool ST, typename TS, typename TC>
-int singles_groups(sci_ctx *ctx, const Tabs &T, const TC *C, typename AccOf<TS>::type *S, int nvec)
+int singles_groups(sci_ctx *ctx, const Tabs &T, const TC *C, typename AccOf<TS>::type *S, int nvec, bool &chained)
 {
     int rc = SCI_OK;
     for (int v0 = 0; v0 < nvec && rc == SCI_OK;) {
         int left = nvec - v0;
         int g = left >= 4 ? 4 : left >= 2 ? 2 : 1;
         switch (g) {
-        case 4: rc = launch_singles<RG, ST, TS, TC, 4>(ctx, T, C, S, nvec, v0); break;
-        case 2: rc = launch_singles<RG, ST, TS, TC, 2>(ctx, T, C, S, nvec, v0); break;
-        default: rc = launch_singles<RG, ST, TS, TC, 1>(ctx, T, C, S, nvec, v0); break;
+        case 4: rc = launch_singles<RG, ST, TS, TC, 4>(ctx, T, C, S, nvec, v0, chained); break;
+        case 2: rc = launch_singles<RG, ST, TS, TC, 2>(ctx, T, C, S, nvec, v0, chained); break;
+        default: rc = launch_singles<RG, ST, TS, TC, 1>(ctx, T, C, S, nvec, v0, chained); break;
         }
         v0 += g;
     }
@@ -1406,12 +1619,6 @@ inline void mark(sci_ctx *ctx, int i)
 }
 
 }  // namespace
-
-#define SCI_CK(call)                                                 \
-    do {                                                             \
-        int _rc = sci_cuda_check(ctx, (call), #call);                \
-        if (_rc != SCI_OK) return _rc;                               \
-    } while (0)
 
 // whether the largest (N-2) bucket fits the staging window of a one-vector launch in the
 // context's scalar mode, row-range launches included (wider vector groups shrink until
@@ -1542,6 +1749,7 @@ int launch_sigma(sci_ctx *ctx, const Tabs &T, const void *C, void *S_out, int nv
     cudaStream_t st = ctx->stream;
     const int64_t row0 = T.rr.rb, nrows = T.rr.re - T.rr.rb;
     int rc;
+    bool chained = false;   // whether a launch of the FP64 chain precedes
     mark(ctx, 0);
     if (ctx->cplx) {
         const zdbl *Cz = (const zdbl *)C;
@@ -1551,11 +1759,11 @@ int launch_sigma(sci_ctx *ctx, const Tabs &T, const void *C, void *S_out, int nv
         SCI_CK(cudaGetLastError());
         mark(ctx, 1);
         rc = prec == SCI_PREC_F64_DS ? ds_groups<RG, ST, true>(ctx, T, C, S, nvec)
-                                     : sigma_groups<RG, ST, zdbl, zdbl>(ctx, T, (const zdbl *)ctx->tab, Cz, Sz, nvec);
+                                     : sigma_groups<RG, ST, zdbl, zdbl>(ctx, T, (const zdbl *)ctx->tab, Cz, Sz, nvec, chained);
         mark(ctx, 2);
         if (rc == SCI_OK)
             rc = prec == SCI_PREC_F64_DS ? ds_singles_groups<RG, ST, true>(ctx, T, C, S1, nvec)
-                                         : singles_groups<RG, ST, zdbl, zdbl>(ctx, T, Cz, (zdbl *)S1, nvec);
+                                         : singles_groups<RG, ST, zdbl, zdbl>(ctx, T, Cz, (zdbl *)S1, nvec, chained);
         mark(ctx, 3);
         if (ST && rc == SCI_OK) rc = row_sums<zdbl, zdbl>(ctx, Cz, (zdbl *)S_out, nvec);
         mark(ctx, 4);
@@ -1570,11 +1778,11 @@ int launch_sigma(sci_ctx *ctx, const Tabs &T, const void *C, void *S_out, int nv
         SCI_CK(cudaGetLastError());
         mark(ctx, 1);
         rc = prec == SCI_PREC_F64_DS ? ds_groups<RG, ST, false>(ctx, T, C, S, nvec)
-                                     : sigma_groups<RG, ST, double, double>(ctx, T, (const double *)ctx->tab, Cd, Sd, nvec);
+                                     : sigma_groups<RG, ST, double, double>(ctx, T, (const double *)ctx->tab, Cd, Sd, nvec, chained);
         mark(ctx, 2);
         if (rc == SCI_OK)
             rc = prec == SCI_PREC_F64_DS ? ds_singles_groups<RG, ST, false>(ctx, T, C, S1, nvec)
-                                         : singles_groups<RG, ST, double, double>(ctx, T, Cd, (double *)S1, nvec);
+                                         : singles_groups<RG, ST, double, double>(ctx, T, Cd, (double *)S1, nvec, chained);
         mark(ctx, 3);
         if (ST && rc == SCI_OK) rc = row_sums<double, double>(ctx, Cd, (double *)S_out, nvec);
         mark(ctx, 4);
