@@ -103,6 +103,7 @@ using sci::col_code;
 using sci::kSmallBucket;
 using sci::kSortBucket;
 using sci::disjoint;
+using sci::doubles_mask;
 using sci::row_code;
 using sci::window;
 
@@ -436,23 +437,6 @@ template <class P, int NV> __device__ __forceinline__ int64_t coef(int64_t I, in
 }
 
 // ------------------------------------------------------------------ walking a row's doubles
-// The doubles of a row among `n` <= 32 consecutive staged members, as a bit mask: bit u is
-// set when member u shares no extra orbital with the row (rc: row_code of the row; code:
-// the members' col_code words).  The row itself and its single excitations leave a 0.
-__device__ __forceinline__ uint32_t doubles_mask(uint32_t rc, const uint32_t *code, int n)
-{
-    uint32_t m = 0;
-    int u = 0;
-    for (; u + 4 <= n; u += 4) {
-        uint32_t g = 0;
-#pragma unroll
-        for (int k = 0; k < 4; k++) g |= (uint32_t)disjoint(rc, code[u + k]) << k;
-        m |= g << u;
-    }
-    for (; u < n; u++) m |= (uint32_t)disjoint(rc, code[u]) << u;
-    return m;
-}
-
 // acc += sum over the set bits u of m of H(row, u) c_u: the pair-table loads of four members
 // are issued before their products, and a member that is no double costs nothing.
 template <class P, int NV>
@@ -579,7 +563,6 @@ k_doubles_sorted(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict_
     for (int k = 0; k < kSortRounds; k++) {
         const int q = wid * per + 32 * k + lane;
         key[k] = -1;
-        rank[k] = 0;
         if (pos[k] != 0) {
             const int size = sci::pos_size(pos[k]), bs = q - sci::pos_off(pos[k]);
             const uint32_t cc = s_code[q];
@@ -599,40 +582,10 @@ k_doubles_sorted(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict_
                 for (int v = 0; v < NV; v++) Sout[(int64_t)slot[r0 + q] * nvec + v0 + v] = typename P::TO{};
             }
         }
-        const unsigned act = __ballot_sync(0xffffffffu, key[k] >= 0);
-        unsigned same = 0;
-        if (key[k] >= 0) {
-            same = __match_any_sync(act, key[k]);
-            rank[k] = s_hist[wid][key[k]] + __popc(same & ((1u << lane) - 1u));
-        }
-        __syncwarp();
-        if (key[k] >= 0 && (same >> lane) == 1u) s_hist[wid][key[k]] = (uint16_t)(rank[k] + 1);   // last of its bin
-        __syncwarp();
+        rank[k] = sci::sort_rank(key[k], s_hist[wid], lane);
     }
     __syncthreads();
-    if (wid == 0) {   // exclusive prefix over (bin, warp); lane l owns bins 2l and 2l + 1
-        int tot[2];
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            int run = 0;
-#pragma unroll
-            for (int w = 0; w < kWarps; w++) {
-                const int c = s_hist[w][2 * lane + h];
-                s_hist[w][2 * lane + h] = (uint16_t)run;
-                run += c;
-            }
-            tot[h] = run;
-        }
-        int inc = tot[0] + tot[1];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += v;
-        }
-        s_base[2 * lane] = inc - tot[0] - tot[1];
-        s_base[2 * lane + 1] = inc - tot[1];
-        if (lane == 31) s_total = inc;
-    }
+    if (wid == 0) sci::sort_prefix<kWarps>(s_hist, lane, s_base, s_total);
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < kSortRounds; k++)
