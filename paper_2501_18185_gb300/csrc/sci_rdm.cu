@@ -58,6 +58,11 @@ __device__ __forceinline__ void mac(zdbl &a, zdbl x, zdbl y)
     a.x = fma(x.x, y.x, fma(-x.y, y.y, a.x));
     a.y = fma(x.x, y.y, fma(x.y, y.x, a.y));
 }
+__device__ __forceinline__ double mul(double x, double y) { return x * y; }
+__device__ __forceinline__ zdbl mul(zdbl x, zdbl y)
+{
+    return zdbl{fma(x.x, y.x, -x.y * y.y), fma(x.x, y.y, x.y * y.x)};
+}
 __device__ __forceinline__ void red(double *p, double v) { atomicAdd(p, v); }
 __device__ __forceinline__ void red(zdbl *p, zdbl v)
 {
@@ -100,9 +105,15 @@ template <int KW> __device__ __forceinline__ bool occ(const Str<KW> &s, int p)
 using sci::RefW;   // the reference string over all words
 
 // Diagonal class: O[p][r] = sum_I w_I n_p n_r in the reference decomposition n = n_ref + d
-// (d = key ^ ref has a few bits), accumulated per CTA in shared memory ([norb]^2 doubles,
-// dynamic: up to 226 KB, 168 spin-orbitals) when SM, else straight into DD and D in
-// global memory (more orbitals).
+// (d = key ^ ref has a few bits, +1 on particles and -1 on holes), accumulated per CTA in
+// shared memory ([norb]^2 doubles, dynamic: up to 226 KB, 168 spin-orbitals) when SM, else
+// straight into DD and D in global memory (more orbitals).  Only DD[p][r] with p < r is kept;
+// DD[p][p] = sum w d_p^2 is D[p] up to the sign of d_p.
+//
+// An FP64 add to shared memory is a compare-and-swap loop, and neighbouring determinants
+// differ from the reference on the same orbitals.  So a warp takes its 32 determinants one
+// after another, its lanes on the (p, r) pairs of one of them, all different addresses.
+// 30 orbitals, M = 250k: a determinant per thread 399 us, a determinant per warp 149 us.
 template <typename TC, int KW, bool SM = true>
 __global__ void __launch_bounds__(kThreads)
 k_rdm_diag(const uint64_t *__restrict__ keys, int64_t M, int norb, RefW ref,
@@ -111,42 +122,59 @@ k_rdm_diag(const uint64_t *__restrict__ keys, int64_t M, int norb, RefW ref,
 {
     extern __shared__ double s_dyn[];
     __shared__ double s_wsum[kThreads / 32];
-    double *sDD = SM ? s_dyn : DD, *sD = SM ? s_dyn + norb * norb : D, *sW = s_wsum;
+    __shared__ uint8_t s_orb[kThreads / 32][64 * KW];   // orbitals of a determinant outside the reference or missing
+    double *sDD = SM ? s_dyn : DD, *sD = SM ? s_dyn + norb * norb : D;
     if constexpr (SM) {
         for (int i = threadIdx.x; i < norb * norb; i += blockDim.x) sDD[i] = 0.0;
         for (int i = threadIdx.x; i < norb; i += blockDim.x) sD[i] = 0.0;
         __syncthreads();
     }
-    Str<KW> rs;
-#pragma unroll
-    for (int k = 0; k < KW; k++) rs.w[k] = ref.w[k];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint8_t *orb = s_orb[wid];
     double wsum = 0.0;
-    for (int64_t I = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; I < M; I += (int64_t)gridDim.x * blockDim.x) {
-        double w = 0.0;
-        for (int v = 0; v < nv; v++) w = fma(wk[v0 + v], sqnorm(C[I * nvec + v0 + v]), w);
-        wsum += w;
-        const Str<KW> key = load_str<KW>(keys, I);
+    for (int64_t I0 = blockIdx.x * (int64_t)blockDim.x + 32 * wid; I0 < M; I0 += (int64_t)gridDim.x * blockDim.x) {
+        const int cnt = (int)min((int64_t)32, M - I0);
+        double wl = 0.0;
+        Str<KW> mine{};
+        if (lane < cnt) {
+            const int64_t I = I0 + lane;
+            for (int v = 0; v < nv; v++) wl = fma(wk[v0 + v], sqnorm(C[I * nvec + v0 + v]), wl);
+            mine = load_str<KW>(keys, I);
+        }
+        wsum += wl;
+        for (int u = 0; u < cnt; u++) {
+            const double w = __shfl_sync(0xffffffffu, wl, u);
+            int nd = 0;
 #pragma unroll
-        for (int k1 = 0; k1 < KW; k1++)
-            for (uint64_t m = key.w[k1] ^ rs.w[k1]; m; m &= m - 1) {
-                const int p = 64 * k1 + __ffsll((long long)m) - 1;
-                const double wp = occ(key, p) ? w : -w;
-                atomicAdd(&sD[p], wp);
+            for (int k = 0; k < KW; k++) {
+                const uint64_t m = __shfl_sync(0xffffffffu, (unsigned long long)mine.w[k], u) ^ ref.w[k];
 #pragma unroll
-                for (int k2 = 0; k2 < KW; k2++)
-                    for (uint64_t m2 = key.w[k2] ^ rs.w[k2]; m2; m2 &= m2 - 1) {
-                        const int r = 64 * k2 + __ffsll((long long)m2) - 1;
-                        atomicAdd(&sDD[p * norb + r], occ(key, r) ? wp : -wp);
-                    }
+                for (int h = 0; h < 2; h++) {
+                    const uint32_t mh = (uint32_t)(m >> (32 * h));
+                    if ((mh >> lane) & 1u) orb[nd + __popc(mh & ((1u << lane) - 1u))] = (uint8_t)(64 * k + 32 * h + lane);
+                    nd += __popc(mh);
+                }
             }
+            __syncwarp();
+            for (int t = lane; t < nd * (nd + 1) / 2; t += 32) {   // t = b(b+1)/2 + a, a <= b
+                int b = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+                while (b * (b + 1) / 2 > t) b--;
+                while ((b + 1) * (b + 2) / 2 <= t) b++;
+                const int p = orb[t - b * (b + 1) / 2], r = orb[b];
+                const bool hp = (ref.w[p >> 6] >> (p & 63)) & 1, hr = (ref.w[r >> 6] >> (r & 63)) & 1;
+                if (p == r) atomicAdd(&sD[p], sflip(hp, w));
+                else atomicAdd(&sDD[p * norb + r], sflip(hp != hr, w));
+            }
+            __syncwarp();
+        }
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, off);
-    if ((threadIdx.x & 31) == 0) sW[threadIdx.x >> 5] = wsum;
+    if (lane == 0) s_wsum[wid] = wsum;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int i = 0; i < kThreads / 32; i++) t += sW[i];
+        for (int i = 0; i < kThreads / 32; i++) t += s_wsum[i];
         atomicAdd(Wt, t);
     }
     if constexpr (SM) {
@@ -157,7 +185,16 @@ k_rdm_diag(const uint64_t *__restrict__ keys, int64_t M, int norb, RefW ref,
     }
 }
 
+// ------------------------------------------------------------------ pairs of a bucket
+// Each unordered pair of a bucket of size s is walked once, with balanced work per row: the
+// member at position q takes the members at q + d (mod s) for d = 1 .. ahead(q, s), which is
+// (s-1)/2, and for even s one more in the first half of the bucket.  The orientation of a
+// pair does not matter: the expansion adds both orientations.
+__device__ __forceinline__ int ahead(int q, int s) { return (s - 1) / 2 + ((s & 1) == 0 && q < s / 2 ? 1 : 0); }
+
 // ------------------------------------------------------------------ singles
+// Bound by the FP64 atomic adds, 2 x level + 2 a pair, so a pair is walked once and not in both
+// orders (30 orbitals, M = 250k, four vectors: 281 -> 148 us).
 template <typename TC, int NV, int KW>
 __global__ void __launch_bounds__(kThreads)
 k_rdm_singles(const uint32_t *__restrict__ e_idx, const uint64_t *__restrict__ e_S, const uint32_t *__restrict__ e_meta,
@@ -168,8 +205,8 @@ k_rdm_singles(const uint32_t *__restrict__ e_idx, const uint64_t *__restrict__ e
         const uint32_t meta = e_meta[p];
         const int x = sci::meta_x(meta);
         const bool par = sci::meta_par(meta);
-        const int64_t bs = p - (int64_t)sci::meta_off(meta);
-        const int64_t be = bs + (int64_t)sci::meta_size(meta);
+        const int off = sci::meta_off(meta), size = sci::meta_size(meta), na = ahead(off, size);
+        if (na == 0) continue;
         // the spectator string's orbitals outside (part) and missing from (holes) the
         // reference, per word
         uint64_t part[KW], holes[KW];
@@ -182,8 +219,8 @@ k_rdm_singles(const uint32_t *__restrict__ e_idx, const uint64_t *__restrict__ e
         TC rowc[NV];
 #pragma unroll
         for (int v = 0; v < NV; v++) rowc[v] = scale(conjv(sflip(par, C[idx * nvec + v0 + v])), wk[v0 + v]);
-        for (int64_t q = bs; q < be; q++) {
-            if (q == p) continue;
+        for (int d = 1; d <= na; d++) {
+            const int64_t q = p + d - (off + d >= size ? size : 0);
             const uint32_t mq = e_meta[q];
             const int y = sci::meta_x(mq);
             const bool parq = sci::meta_par(mq);
@@ -205,142 +242,316 @@ k_rdm_singles(const uint32_t *__restrict__ e_idx, const uint64_t *__restrict__ e
 }
 
 // ------------------------------------------------------------------ doubles
-// Each unordered pair of a bucket of size s is walked once, with balanced work per lane:
-// the member at position q takes the members at q + d (mod s) for d = 1 .. (s-1)/2, and
-// for even s the member at distance s/2 is taken by the first half of the bucket.  The
-// orientation of a pair does not matter: the expansion adds both orientations.
+// A pair costs NV FP64 FMAs and one FP64 atomic add to the L2, and the FP64 pipe binds (a warp
+// instruction holds it 16 cycles whatever its active lanes).  So the rows find their doubles
+// first, as bit masks, and issue FP64 work for doubles only; by bucket size (entries are
+// ordered by it, as in sigma): above kSortBucket members k_rdm_doubles, whose rows walk whole
+// buckets and have similar counts; 5 to 64 k_rdm_doubles_sorted, rows sorted by their count;
+// up to 4 k_rdm_doubles_small, in registers.
+// 30 orbitals, M = 250k, four vectors: all sizes in one walk member by member 1.11 ms; 0.93 by
+// size (above 64 members 0.49 ms, 5 to 64 0.35, up to 4 0.09).
+constexpr int kMaskWords = 4;   // members per pass of a row over its bucket: 128
+
 template <typename TC, int NV>
 __global__ void __launch_bounds__(kThreads)
 k_rdm_doubles(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict__ e_code, const uint32_t *__restrict__ e_pos,
               int64_t E, int CH, sci::TabRule tr, uint32_t bb_off, const TC *__restrict__ C, int nvec, int v0,
               const double *__restrict__ wk, TC *__restrict__ dT)
 {
-    constexpr int nv = NV;
     extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t s_mask[kMaskWords][kThreads];   // a column per thread, no barrier needed
     int64_t r0, r1;
     sci::window(e_pos, E, CH, r0, r1);
     if (r0 >= r1) return;
     const int W = (int)(r1 - r0);
-    TC *s_c = reinterpret_cast<TC *>(smem);  // [W][nv]: c of each member times (-1)^pi
-    const size_t cbytes = ((size_t)W * nv * sizeof(TC) + 15) & ~(size_t)15;
-    uint2 *s_kc = reinterpret_cast<uint2 *>(smem + cbytes);
+    TC *s_c = reinterpret_cast<TC *>(smem);  // [W][NV]: c of each member times (-1)^pi
+    uint32_t *s_code = reinterpret_cast<uint32_t *>(s_c + (size_t)W * NV), *s_col = s_code + W;
     for (int q = threadIdx.x; q < W; q += blockDim.x) {
         const int64_t g = r0 + q;
         const uint32_t code = e_code[g];
         const int64_t idx = e_idx[g];
         uint32_t rowoff, colbase;
         grad_offsets(tr, sci::code_x(code), sci::code_y(code), bb_off, rowoff, colbase);
-        s_kc[q] = make_uint2(sci::col_code(code), colbase);
+        s_code[q] = sci::col_code(code);
+        s_col[q] = colbase;
         const bool par = sci::code_par(code);
-        for (int v = 0; v < nv; v++) s_c[q * nv + v] = sflip(par, C[idx * nvec + v0 + v]);
+        for (int v = 0; v < NV; v++) s_c[q * NV + v] = sflip(par, C[idx * nvec + v0 + v]);
     }
     __syncthreads();
     for (int q0 = threadIdx.x; q0 < W; q0 += blockDim.x) {
         const uint32_t code = e_code[r0 + q0], pos = e_pos[r0 + q0];
         uint32_t rowoff, colbase;
         grad_offsets(tr, sci::code_x(code), sci::code_y(code), bb_off, rowoff, colbase);
-        const int qp = sci::pos_off(pos), sz = sci::pos_size(pos), bs = q0 - qp;
-        const int dmax = (sz - 1) / 2 + ((sz & 1) == 0 && qp < sz / 2 ? 1 : 0);
+        const int qp = sci::pos_off(pos), sz = sci::pos_size(pos), bs = q0 - qp, be = bs + sz;
         const uint32_t rc = sci::row_code(code);
         TC rowc[NV];
 #pragma unroll
-        for (int v = 0; v < NV; v++) rowc[v] = scale(conjv(s_c[q0 * nv + v]), wk[v0 + v]);
+        for (int v = 0; v < NV; v++) rowc[v] = scale(conjv(s_c[q0 * NV + v]), wk[v0 + v]);
         TC *trow = dT + rowoff;
-        int j = qp;
-        for (int d = 1; d <= dmax; d++) {
-            j = j + 1 == sz ? 0 : j + 1;
-            const uint2 kc = s_kc[bs + j];
-            if (!sci::disjoint(rc, kc.x)) continue;
-            TC w;
-            zero(w);
+        int at = q0 + 1, left = ahead(qp, sz);   // at: window row of the next member, before wrapping
+        for (; left > 0; at += 32 * kMaskWords, left -= 32 * kMaskWords) {
+            int n = 0;
+            for (int w = 0; w < kMaskWords && 32 * w < left; w++) {
+                const int j0 = at + 32 * w, len = min(32, left - 32 * w);
+                // the members before and after the wrap to the start of the bucket
+                const int first = min(max(be - j0, 0), len);
+                uint32_t m = sci::doubles_mask(rc, s_code + j0, first);
+                if (first < len) m |= sci::doubles_mask(rc, s_code + (j0 + first - sz), len - first) << first;
+                s_mask[w][threadIdx.x] = m;
+                n += __popc(m);
+            }
+            int w = -1;
+            uint32_t m = 0;
+            for (; n > 0; n--) {
+                while (m == 0) m = s_mask[++w][threadIdx.x];
+                int j = at + 32 * w + __ffs((int)m) - 1;
+                m &= m - 1;
+                j = j >= be ? j - sz : j;
+                TC sum = mul(rowc[0], s_c[j * NV]);
 #pragma unroll
-            for (int v = 0; v < NV; v++) mac(w, rowc[v], s_c[(bs + j) * nv + v]);
-            red(trow + kc.y, w);
+                for (int v = 1; v < NV; v++) mac(sum, rowc[v], s_c[j * NV + v]);
+                red(trow + s_col[j], sum);
+            }
         }
     }
+}
+
+// Buckets of at most kSortBucket members.  A CTA owns the whole buckets that start in its
+// kSortRows table rows; the doubles ahead of a row are a 64-bit mask, and the rows are sorted
+// by their count, so that the lanes of a warp stay on useful products.  Members without any
+// double read no coefficients.
+constexpr int kSortRows = 448;
+constexpr int kSortCap = kSortRows + sci::kSortBucket;   // rows of a window, at most
+constexpr int kSortRounds = kSortCap / kThreads;
+static_assert(kSortCap % kThreads == 0, "every thread holds the same number of rows");
+
+template <typename TC, int NV> constexpr size_t sort_smem()
+{
+    return (size_t)kSortCap * (NV * sizeof(TC) + sizeof(uint64_t) + 3 * sizeof(uint32_t));
+}
+
+template <typename TC, int NV>
+__global__ void __launch_bounds__(kThreads)
+k_rdm_doubles_sorted(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict__ e_code,
+                     const uint32_t *__restrict__ e_pos, int64_t E, sci::TabRule tr, uint32_t bb_off,
+                     const TC *__restrict__ C, int nvec, int v0, const double *__restrict__ wk, TC *__restrict__ dT)
+{
+    constexpr int kWarps = kThreads / 32;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint16_t s_hist[kWarps][64];
+    __shared__ int s_base[64], s_total;
+    int64_t r0, r1;
+    sci::window(e_pos, E, kSortRows, r0, r1);
+    if (r0 >= r1) return;
+    const int W = (int)(r1 - r0);
+    TC *s_c = reinterpret_cast<TC *>(smem);
+    uint64_t *s_mask = reinterpret_cast<uint64_t *>(s_c + kSortCap * NV);
+    uint32_t *s_code = reinterpret_cast<uint32_t *>(s_mask + kSortCap);
+    uint32_t *s_col = s_code + kSortCap;
+    uint32_t *s_row = s_col + kSortCap;    // sorted rows: window row | bucket position << 16
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // warp w holds the rows [w * per, (w + 1) * per), 32 at a time
+    const int per = ((W + kWarps - 1) / kWarps + 31) & ~31;
+
+    uint32_t pos[kSortRounds];
+    bool par[kSortRounds];
+#pragma unroll
+    for (int k = 0; k < kSortRounds; k++) {
+        const int q = wid * per + 32 * k + lane;
+        pos[k] = 0;
+        par[k] = false;
+        if (32 * k < per && q < W) {
+            const uint32_t code = e_code[r0 + q];
+            pos[k] = e_pos[r0 + q];
+            par[k] = sci::code_par(code);
+            uint32_t rowoff, colbase;
+            grad_offsets(tr, sci::code_x(code), sci::code_y(code), bb_off, rowoff, colbase);
+            s_code[q] = sci::col_code(code);
+            s_col[q] = colbase;
+        }
+    }
+    for (int t = threadIdx.x; t < kWarps * 64; t += kThreads) (&s_hist[0][0])[t] = 0;
+    __syncthreads();
+
+    int key[kSortRounds], rank[kSortRounds];
+#pragma unroll
+    for (int k = 0; k < kSortRounds; k++) {
+        const int q = wid * per + 32 * k + lane;
+        key[k] = -1;
+        if (pos[k] != 0) {
+            const int size = sci::pos_size(pos[k]), qp = sci::pos_off(pos[k]), bs = q - qp;
+            const uint32_t rc = __byte_perm(s_code[q], 0, 0x1010);   // (x, y, x, y) of the row
+            uint64_t m = sci::doubles_mask(rc, s_code + bs, min(size, 32));
+            if (size > 32) m |= (uint64_t)sci::doubles_mask(rc, s_code + bs + 32, size - 32) << 32;
+            if (m) {
+                const int64_t I = e_idx[r0 + q];
+#pragma unroll
+                for (int v = 0; v < NV; v++) s_c[q * NV + v] = sflip(par[k], C[I * nvec + v0 + v]);
+            }
+            // the members ahead of the row, cyclically: bits qp + 1 .. qp + ahead (mod size)
+            const uint64_t a = (1ull << ahead(qp, size)) - 1;
+            const uint64_t window = (qp < 63 ? a << (qp + 1) : 0ull) | a >> (size - qp - 1);
+            m &= window;   // bits from `size` on are no members and not set in m
+            s_mask[q] = m;
+            if (m) key[k] = 32 - __popcll(m);
+        }
+        rank[k] = sci::sort_rank(key[k], s_hist[wid], lane);
+    }
+    __syncthreads();
+    if (wid == 0) sci::sort_prefix<kWarps>(s_hist, lane, s_base, s_total);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kSortRounds; k++)
+        if (key[k] >= 0) {
+            const int q = wid * per + 32 * k + lane;
+            s_row[s_base[key[k]] + s_hist[wid][key[k]] + rank[k]] = (uint32_t)q | (uint32_t)sci::pos_off(pos[k]) << 16;
+        }
+    __syncthreads();
+
+    const int nrows = s_total;
+    for (int t = threadIdx.x; t < nrows; t += kThreads) {
+        const uint32_t row = s_row[t];
+        const int q = (int)(row & 0xFFFFu), bs = q - (int)(row >> 16);
+        const uint32_t cc = s_code[q];
+        uint32_t rowoff, colbase;
+        grad_offsets(tr, (int)(cc & 0xFFu), (int)((cc >> 8) & 0xFFu), bb_off, rowoff, colbase);
+        TC rowc[NV];
+#pragma unroll
+        for (int v = 0; v < NV; v++) rowc[v] = scale(conjv(s_c[q * NV + v]), wk[v0 + v]);
+        TC *trow = dT + rowoff;
+        for (uint64_t m = s_mask[q]; m; m &= m - 1) {
+            const int j = bs + __ffsll((long long)m) - 1;
+            TC sum = mul(rowc[0], s_c[j * NV]);
+#pragma unroll
+            for (int v = 1; v < NV; v++) mac(sum, rowc[v], s_c[j * NV + v]);
+            red(trow + s_col[j], sum);
+        }
+    }
+}
+
+// Buckets of S <= kSmallBucket members: most entries of a selected space, few of its pairs.  A
+// thread takes a bucket, its members in registers; members without a double read nothing.
+template <typename TC, int S, int NV>
+__global__ void __launch_bounds__(kThreads)
+k_rdm_doubles_small(const uint32_t *__restrict__ e_idx, const uint32_t *__restrict__ e_code, int64_t nbuckets,
+                    sci::TabRule tr, uint32_t bb_off, const TC *__restrict__ C, int nvec, int v0,
+                    const double *__restrict__ wk, TC *__restrict__ dT)
+{
+    const int64_t b = blockIdx.x * (int64_t)kThreads + threadIdx.x;
+    if (b >= nbuckets) return;
+    const int64_t g = b * S;
+    uint32_t code[S], col[S];
+    int64_t idx[S];
+#pragma unroll
+    for (int i = 0; i < S; i++) code[i] = e_code[g + i];
+    bool any = false, dbl[S][S];
+#pragma unroll
+    for (int i = 0; i < S; i++)
+#pragma unroll
+        for (int j = 0; j < i; j++) {
+            dbl[i][j] = sci::disjoint(sci::row_code(code[i]), sci::col_code(code[j]));
+            any |= dbl[i][j];
+        }
+    if (!any) return;
+    uint32_t row[S];
+#pragma unroll
+    for (int i = 0; i < S; i++) {
+        idx[i] = e_idx[g + i];
+        grad_offsets(tr, sci::code_x(code[i]), sci::code_y(code[i]), bb_off, row[i], col[i]);
+    }
+    TC sum[S][S];
+#pragma unroll
+    for (int v = 0; v < NV; v++) {
+        TC c[S];
+#pragma unroll
+        for (int i = 0; i < S; i++) c[i] = sflip(sci::code_par(code[i]), C[idx[i] * nvec + v0 + v]);
+#pragma unroll
+        for (int i = 1; i < S; i++) {
+            const TC r = scale(conjv(c[i]), wk[v0 + v]);
+#pragma unroll
+            for (int j = 0; j < i; j++)
+                if (dbl[i][j]) {
+                    if (v == 0) sum[i][j] = mul(r, c[j]);
+                    else mac(sum[i][j], r, c[j]);
+                }
+        }
+    }
+#pragma unroll
+    for (int i = 1; i < S; i++)
+#pragma unroll
+        for (int j = 0; j < i; j++)
+            if (dbl[i][j]) red(dT + row[i] + col[j], sum[i][j]);
 }
 
 // ------------------------------------------------------------------ expansion
-// g1 and the g2 elements of the diagonal and single-excitation classes; one thread per
-// (x, y)
-// occupation of orbital k in the reference
-__device__ __forceinline__ double ref_occ(const RefW &ref, int k) { return (double)((ref.w[k >> 6] >> (k & 63)) & 1); }
+// The elements of g1 and g2 from the tables of the three classes.
+template <typename TC> struct Tables {
+    sci::TabRule tr;
+    int norb;
+    uint32_t bb_off;
+    RefW ref;
+    const double *Wt, *D, *DD;
+    const TC *A, *Bc, *dT;
 
-template <typename TC>
-__global__ void k_rdm_expand1(int norb, RefW ref, const double *__restrict__ Wt,
-                              const double *__restrict__ D, const double *__restrict__ DD, const TC *__restrict__ A,
-                              const TC *__restrict__ Bc, TC *__restrict__ g1, TC *__restrict__ g2)
+    __device__ __forceinline__ double occ_ref(int k) const { return (double)((ref.w[k >> 6] >> (k & 63)) & 1); }
+    __device__ __forceinline__ int spin(int p) const { return tr.spinors ? 0 : p >= tr.n; }
+    // sum_I w_I n_x n_y
+    __device__ __forceinline__ double pair_occ(int x, int y) const
+    {
+        const double nx = occ_ref(x), ny = occ_ref(y);
+        const double dd = x == y ? (nx != 0.0 ? -D[x] : D[x]) : DD[min(x, y) * norb + max(x, y)];
+        return *Wt * nx * ny + nx * D[y] + D[x] * ny + dd;
+    }
+    // <a+_x a_y>, x != y
+    __device__ __forceinline__ TC single(int x, int y) const { return add(A[x * norb + y], conjv(A[y * norb + x])); }
+    // <a+_x a_y n_k>, x, y and k different
+    __device__ __forceinline__ TC spectator(int x, int y, int k) const
+    {
+        if (spin(x) != spin(y)) return from_real<TC>(0.0);
+        const TC b = add(Bc[((int64_t)x * norb + y) * norb + k], conjv(Bc[((int64_t)y * norb + x) * norb + k]));
+        return add(scale(single(x, y), occ_ref(k)), b);
+    }
+    // <a+_p a+_r a_s a_q>
+    __device__ __forceinline__ TC two(int p, int q, int r, int s) const
+    {
+        const TC none = from_real<TC>(0.0);
+        if (p == r || q == s) return none;
+        if (p == q) return r == s ? from_real<TC>(pair_occ(p, r)) : spectator(r, s, p);
+        if (r == s) return spectator(p, q, r);
+        if (p == s) return r == q ? from_real<TC>(-pair_occ(p, r)) : neg(spectator(r, q, p));
+        if (r == q) return neg(spectator(p, s, r));
+        if (spin(p) + spin(r) != spin(q) + spin(s)) return none;
+        // a double excitation: both orientations of the pair table
+        uint32_t row, col, row2, col2;
+        grad_offsets(tr, min(p, r), max(p, r), bb_off, row, col2);
+        grad_offsets(tr, min(q, s), max(q, s), bb_off, row2, col);
+        const TC u = add(dT[(int64_t)row + col], conjv(dT[(int64_t)row2 + col2]));
+        return (p < r) == (q < s) ? u : neg(u);
+    }
+};
+
+template <typename TC> __global__ void k_rdm_expand1(Tables<TC> T, TC *__restrict__ g1)
 {
-    const int64_t n2 = (int64_t)norb * norb, n3 = n2 * norb;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n2; t += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(t / norb), y = (int)(t % norb);
-        const double nx = ref_occ(ref, x), ny = ref_occ(ref, y);
-        const double O = *Wt * nx * ny + nx * D[y] + D[x] * ny + DD[t];
-        const TC o = from_real<TC>(O);
-        if (x == y) {
-            g1[t] = o;
-            continue;
-        }
-        const TC a = A[t];
-        g1[t] = a;
-        if (!g2) continue;
-        g2[(int64_t)x * n3 + (int64_t)x * n2 + (int64_t)y * norb + y] = o;         // (x x | y y)
-        g2[(int64_t)x * n3 + (int64_t)y * n2 + (int64_t)y * norb + x] = neg(o);    // (x y | y x)
-        for (int k = 0; k < norb; k++) {
-            if (k == x || k == y) continue;
-            const TC b = add(scale(a, ref_occ(ref, k)), Bc[t * norb + k]);
-            const TC nb = neg(b);
-            g2[(int64_t)x * n3 + (int64_t)y * n2 + (int64_t)k * norb + k] = b;     // (x y | k k)
-            g2[(int64_t)k * n3 + (int64_t)k * n2 + (int64_t)x * norb + y] = b;     // (k k | x y)
-            g2[(int64_t)x * n3 + (int64_t)k * n2 + (int64_t)k * norb + y] = nb;    // (x k | k y)
-            g2[(int64_t)k * n3 + (int64_t)y * n2 + (int64_t)x * norb + k] = nb;    // (k y | x k)
-        }
+    const int n2 = T.norb * T.norb;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n2; t += gridDim.x * blockDim.x) {
+        const int x = t / T.norb, y = t % T.norb;
+        g1[t] = x == y ? from_real<TC>(T.pair_occ(x, x)) : T.single(x, y);
     }
 }
 
-// unordered pair index P(a, b) = b(b-1)/2 + a, a < b -> (a, b)
-__device__ __forceinline__ void unpair(int P, int &a, int &b)
+// g2, every element once in storage order: a CTA takes the [r][s] matrices of its (p, q), so
+// that the writes, which bound it (norb^4 elements, 104 MB at 60 spin-orbitals), are
+// consecutive and g2 needs no clearing; the tables are small and read from L2.
+// 118 us at 60 spin-orbitals, where the clear and the scattered stores of one thread per table
+// entry took 100; the gradients, which sum straight from the tables, no longer form g2.  (Adding
+// the two orientations in a pass of its own first: 122 us for both.)
+template <typename TC> __global__ void __launch_bounds__(kThreads) k_rdm_expand2(Tables<TC> T, TC *__restrict__ g2)
 {
-    int bb = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)P)) * 0.5f);
-    while (bb * (bb - 1) / 2 > P) bb--;
-    while ((bb + 1) * bb / 2 <= P) bb++;
-    b = bb;
-    a = P - bb * (bb - 1) / 2;
-}
-
-// g2 elements of the double-excitation class from the gradient table; one thread per
-// table entry (bra, ket), writing the four elements of that orientation
-template <typename TC>
-__global__ void k_rdm_expand2(sci::TabRule tr, int norb, int64_t nT, const TC *__restrict__ dT, TC *__restrict__ g2)
-{
-    const int n = tr.n;
-    const int64_t n2 = (int64_t)norb * norb, n3 = n2 * norb;
-    const int64_t NP = (int64_t)n * (n - 1) / 2;
-    const int64_t nab = tr.spinors ? 0 : (int64_t)n * n * n * n;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nT; e += (int64_t)gridDim.x * blockDim.x) {
-        int a, b, i, j;
-        int64_t et;
-        if (e < nab) {  // alpha-beta: e = u_ket * n^2 + u_bra, u = (y - n) * n + x
-            const int64_t ub = e % ((int64_t)n * n), uk = e / ((int64_t)n * n);
-            a = (int)(ub % n), b = n + (int)(ub / n);
-            i = (int)(uk % n), j = n + (int)(uk / n);
-            et = ub * ((int64_t)n * n) + uk;
-        } else {        // same spin (spinor mode: all): e = p_ket * NP + p_bra
-            const int64_t e2 = e - nab;
-            const int64_t reg = e2 / (NP * NP), r = e2 % (NP * NP);
-            const int pb = (int)(r % NP), pk = (int)(r / NP);
-            unpair(pb, a, b);
-            unpair(pk, i, j);
-            if (reg) a += n, b += n, i += n, j += n;  // beta-beta region
-            et = nab + reg * (NP * NP) + (int64_t)pb * NP + pk;
-        }
-        if (a == i || a == j || b == i || b == j) continue;  // not a double: other classes own these
-        const TC u = add(dT[e], conjv(dT[et]));
-        const TC nu = neg(u);
-        g2[(int64_t)a * n3 + (int64_t)i * n2 + (int64_t)b * norb + j] = u;
-        g2[(int64_t)b * n3 + (int64_t)j * n2 + (int64_t)a * norb + i] = u;
-        g2[(int64_t)a * n3 + (int64_t)j * n2 + (int64_t)b * norb + i] = nu;
-        g2[(int64_t)b * n3 + (int64_t)i * n2 + (int64_t)a * norb + j] = nu;
+    const int norb = T.norb, n2 = norb * norb;
+    for (int pq = blockIdx.x; pq < n2; pq += gridDim.x) {
+        const int p = pq / norb, q = pq % norb;
+        TC *out = g2 + (int64_t)pq * n2;
+        for (int t = threadIdx.x; t < n2; t += blockDim.x) out[t] = T.two(p, q, t / norb, t % norb);
     }
 }
 
@@ -361,6 +572,15 @@ template <typename TC> struct Walk {
     uint32_t bb_off;
 };
 
+// the buckets of exactly S members
+template <typename TC, int S, int NV> void launch_small(sci_ctx *ctx, const Walk<TC> &w)
+{
+    const int64_t at = ctx->split2.above[S], n = (ctx->split2.above[S - 1] - at) / S;
+    if (n > 0)
+        k_rdm_doubles_small<TC, S, NV><<<(unsigned)((n + kThreads - 1) / kThreads), kThreads, 0, ctx->stream>>>(
+            ctx->e2_idx + at, ctx->e2_code + at, n, w.tr, w.bb_off, w.C, w.nvec, w.v0, w.wk, w.dT);
+}
+
 // the single- and double-excitation walks for one group of NV vectors
 template <typename TC, int NV>
 int launch_walks(sci_ctx *ctx, const Walk<TC> &w)
@@ -374,20 +594,38 @@ int launch_walks(sci_ctx *ctx, const Walk<TC> &w)
                                                             ref_words(ctx), w.C, w.nvec, w.v0, w.wk, w.A, w.Bc);
     }
     if (w.dT) {
-        auto kern = k_rdm_doubles<TC, NV>;
-        if (w.smem > 48 * 1024 &&
-            sci_cuda_check(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w.smem),
-                           "rdm12 attr"))
-            return SCI_ERR_CUDA;
-        const int64_t blocks = (ctx->e2 + w.CH - 1) / w.CH;
-        kern<<<(unsigned)blocks, kThreads, w.smem, ctx->stream>>>(ctx->e2_idx, ctx->e2_code, ctx->e2_pos, ctx->e2, w.CH,
-                                                                 w.tr, w.bb_off, w.C, w.nvec, w.v0, w.wk, w.dT);
+        const int64_t large = ctx->split2.above[sci::kSortBucket], mid = ctx->split2.above[sci::kSmallBucket];
+        if (large > 0) {
+            auto kern = k_rdm_doubles<TC, NV>;
+            if (w.smem > 32 * 1024 &&
+                sci_cuda_check(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w.smem),
+                               "rdm12 attr"))
+                return SCI_ERR_CUDA;
+            kern<<<(unsigned)((large + w.CH - 1) / w.CH), kThreads, w.smem, ctx->stream>>>(
+                ctx->e2_idx, ctx->e2_code, ctx->e2_pos, large, w.CH, w.tr, w.bb_off, w.C, w.nvec, w.v0, w.wk, w.dT);
+        }
+        if (mid > large) {
+            auto kern = k_rdm_doubles_sorted<TC, NV>;
+            constexpr size_t smem = sort_smem<TC, NV>();
+            if (smem > 32 * 1024 &&
+                sci_cuda_check(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                               "rdm12 attr"))
+                return SCI_ERR_CUDA;
+            kern<<<(unsigned)((mid - large + kSortRows - 1) / kSortRows), kThreads, smem, ctx->stream>>>(
+                ctx->e2_idx + large, ctx->e2_code + large, ctx->e2_pos + large, mid - large, w.tr, w.bb_off, w.C,
+                w.nvec, w.v0, w.wk, w.dT);
+        }
+        launch_small<TC, 4, NV>(ctx, w);
+        launch_small<TC, 3, NV>(ctx, w);
+        launch_small<TC, 2, NV>(ctx, w);
     }
     return SCI_OK;
 }
 
+// the class tables of a weighted set of vectors, in the context's scratch; with_two: also the
+// double-excitation table.  C and the weights are device pointers.
 template <typename TC>
-int rdm_run(sci_ctx *ctx, const TC *C, int nvec, const double *wk_dev, TC *g1, TC *g2)
+int rdm_tables(sci_ctx *ctx, const TC *C, int nvec, const double *wk_dev, bool with_two, Tables<TC> &T)
 {
     const int norb = ctx->norb, n = ctx->n;
     const int64_t n2 = (int64_t)norb * norb;
@@ -396,7 +634,7 @@ int rdm_run(sci_ctx *ctx, const TC *C, int nvec, const double *wk_dev, TC *g1, T
     const uint32_t bb_off = ctx->spinors ? 0u : (uint32_t)(NP * NP);
     // scratch: Wt, D[norb], DD[norb^2] (double); A[norb^2], Bc[norb^3], dT[nT] (TC)
     const size_t dbytes = sizeof(double) * (1 + norb + n2);
-    const size_t tbytes = sizeof(TC) * (n2 + n2 * norb + (g2 ? nT : 0));
+    const size_t tbytes = sizeof(TC) * (n2 + n2 * norb + (with_two ? nT : 0));
     const size_t need = ((dbytes + 255) & ~(size_t)255) + tbytes;
     if (need > ctx->rdm_bytes) {
         if (ctx->rdm_scratch) cudaFree(ctx->rdm_scratch);
@@ -409,23 +647,24 @@ int rdm_run(sci_ctx *ctx, const TC *C, int nvec, const double *wk_dev, TC *g1, T
     TC *A = reinterpret_cast<TC *>(base + ((dbytes + 255) & ~(size_t)255));
     TC *Bc = A + n2;
     TC *dT = Bc + n2 * norb;
-    if (sci_cuda_check(ctx, cudaMemsetAsync(ctx->rdm_scratch, 0, need, ctx->stream), "rdm12 memset") ||
-        (g2 && sci_cuda_check(ctx, cudaMemsetAsync(g2, 0, sizeof(TC) * n2 * n2, ctx->stream), "rdm12 memset g2")))
-        return SCI_ERR_CUDA;
+    if (sci_cuda_check(ctx, cudaMemsetAsync(ctx->rdm_scratch, 0, need, ctx->stream), "rdm12 memset")) return SCI_ERR_CUDA;
     const sci::TabRule tr{ctx->spinors, n};
-    const int CH = 768;
+    // window rows of the large buckets: short windows where there are few (shared memory, and
+    // with it the CTAs per SM, is the largest bucket's: 441 members at 30 orbitals;
+    // 1.47M entries of buckets above 64: 546 us at 768 rows, 491 at 256)
+    const int CH = ctx->split2.above[sci::kSortBucket] / 768 >= 152 * 16 ? 768 : 256;
     auto stage_bytes = [&](int nv) {
-        return (((size_t)(CH + ctx->maxb2) * nv * sizeof(TC) + 15) & ~(size_t)15) + (size_t)(CH + ctx->maxb2) * sizeof(uint2);
+        return (size_t)(CH + ctx->maxb2) * (nv * sizeof(TC) + 2 * sizeof(uint32_t));
     };
     // vectors per walk: at most kMaxVec, fewer when the staged window would not fit
     int kv = kMaxVec;
     while (kv > 1 && stage_bytes(kv) > 200 * 1024) kv >>= 1;
-    if (g2 && ctx->e2 > 0 && stage_bytes(kv) > 200 * 1024)
+    if (with_two && ctx->e2 > 0 && stage_bytes(kv) > 200 * 1024)
         return sci_fail(ctx, SCI_ERR_OVERFLOW, "rdm12: largest bucket too large for shared memory");
     // the diagonal kernel: DD [norb]^2 and D [norb] in shared memory while they fit (up to
     // 168 orbitals), else accumulated in global memory
     size_t diag_smem = sizeof(double) * ((size_t)norb * norb + norb);
-    const bool diag_sm = diag_smem + 1024 <= 227 * 1024;
+    const bool diag_sm = diag_smem + 4096 <= 227 * 1024;
     auto kd = ctx->nwords == 4   ? (diag_sm ? k_rdm_diag<TC, 4, true> : k_rdm_diag<TC, 4, false>)
               : ctx->nwords == 3 ? (diag_sm ? k_rdm_diag<TC, 3, true> : k_rdm_diag<TC, 3, false>)
               : ctx->nwords == 2 ? k_rdm_diag<TC, 2, true>
@@ -436,9 +675,9 @@ int rdm_run(sci_ctx *ctx, const TC *C, int nvec, const double *wk_dev, TC *g1, T
         return SCI_ERR_CUDA;
     for (int v0 = 0; v0 < nvec; v0 += kv) {
         const int nv = std::min(kv, nvec - v0);
-        kd<<<grid_for(ctx->M), kThreads, diag_smem, ctx->stream>>>(ctx->keys, ctx->M, norb, ref_words(ctx), C, nvec, v0,
+        kd<<<std::min(grid_for(ctx->M), 152 * 7), kThreads, diag_smem, ctx->stream>>>(ctx->keys, ctx->M, norb, ref_words(ctx), C, nvec, v0,
                                                                    nv, wk_dev, Wt, D, DD);
-        const Walk<TC> wlk{C, nvec, v0, wk_dev, A, Bc, g2 && ctx->e2 > 0 ? dT : nullptr, CH, stage_bytes(nv), tr, bb_off};
+        const Walk<TC> wlk{C, nvec, v0, wk_dev, A, Bc, with_two && ctx->e2 > 0 ? dT : nullptr, CH, stage_bytes(nv), tr, bb_off};
         int rc = SCI_OK;
         switch (nv) {
             case 1: rc = launch_walks<TC, 1>(ctx, wlk); break;
@@ -452,77 +691,105 @@ int rdm_run(sci_ctx *ctx, const TC *C, int nvec, const double *wk_dev, TC *g1, T
         }
         if (rc) return rc;
     }
-    k_rdm_expand1<TC><<<grid_for(n2), kThreads, 0, ctx->stream>>>(norb, ref_words(ctx), Wt, D, DD, A, Bc, g1, g2);
-    if (g2) k_rdm_expand2<TC><<<grid_for(nT), kThreads, 0, ctx->stream>>>(tr, norb, nT, dT, g2);
+    T = Tables<TC>{tr, norb, bb_off, ref_words(ctx), Wt, D, DD, A, Bc, dT};
+    return SCI_OK;
+}
+
+template <typename TC>
+int rdm_run(sci_ctx *ctx, const TC *C, int nvec, const double *wk_dev, TC *g1, TC *g2)
+{
+    Tables<TC> T;
+    const int rc = rdm_tables<TC>(ctx, C, nvec, wk_dev, g2 != nullptr, T);
+    if (rc) return rc;
+    const int n2 = ctx->norb * ctx->norb;
+    k_rdm_expand1<TC><<<grid_for(n2), kThreads, 0, ctx->stream>>>(T, g1);
+    if (g2) k_rdm_expand2<TC><<<n2, kThreads, 0, ctx->stream>>>(T, g2);
     return sci_cuda_check(ctx, cudaGetLastError(), "rdm12 launch") ? SCI_ERR_CUDA : SCI_OK;
+}
+
+// the weights of a call (a host array of nvec doubles, NULL = all ones) on the device
+int rdm_weights(sci_ctx *ctx, int nvec, const double *weights)
+{
+    const size_t wbytes = sizeof(double) * nvec;
+    if (wbytes > ctx->rdm_wbytes) {
+        if (ctx->rdm_w) cudaFree(ctx->rdm_w);
+        ctx->rdm_w = nullptr, ctx->rdm_wbytes = 0;
+        if (cudaMalloc(&ctx->rdm_w, wbytes) != cudaSuccess) return sci_fail(ctx, SCI_ERR_NOMEM, "rdm12: weights");
+        ctx->rdm_wbytes = wbytes;
+    }
+    std::vector<double> w(nvec, 1.0);
+    if (weights) std::copy(weights, weights + nvec, w.begin());
+    if (sci_cuda_check(ctx, cudaMemcpyAsync(ctx->rdm_w, w.data(), wbytes, cudaMemcpyHostToDevice, ctx->stream), "rdm12 weights") ||
+        sci_cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "rdm12 weights sync"))
+        return SCI_ERR_CUDA;
+    return SCI_OK;
 }
 
 // ------------------------------------------------------------------ gradients of E
 // Spin sums of the spin-orbital density matrices (bit p < n alpha p, bit n + p beta p):
 //   gamma[p][q]        = sum_s g1[ps][qs]
 //   Gamma[p][q][r][s]  = sum_{s1,s2} g2[p s1][q s1][r s2][s s2]
-__global__ void k_spin_sum1(int n, const double *__restrict__ g1, double *__restrict__ gamma)
+__global__ void k_spin_sum1(int n, Tables<double> T, double *__restrict__ gamma)
 {
-    const int norb = 2 * n;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n * n; t += gridDim.x * blockDim.x) {
         const int p = t / n, q = t % n;
-        gamma[t] = g1[p * norb + q] + g1[(n + p) * norb + n + q];
+        gamma[t] = p == q ? T.pair_occ(p, p) + T.pair_occ(n + p, n + p) : T.single(p, q) + T.single(n + p, n + q);
     }
 }
 
-__global__ void k_spin_sum2(int n, const double *__restrict__ g2, double *__restrict__ Gamma)
+// straight from the class tables: the spin-orbital g2, sixteen times Gamma, is never formed
+__global__ void k_spin_sum2(int n, Tables<double> T, double *__restrict__ Gamma)
 {
-    const int64_t norb = 2 * n, n4 = (int64_t)n * n * n * n;
+    const int64_t n4 = (int64_t)n * n * n * n;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n4; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t s = t % n, r = (t / n) % n, q = (t / n / n) % n, p = t / n / n / n;
+        const int s = (int)(t % n), r = (int)((t / n) % n), q = (int)((t / n / n) % n), p = (int)(t / n / n / n);
         double v = 0.0;
         for (int a = 0; a < 2; a++)
-            for (int b = 0; b < 2; b++)
-                v += g2[(((p + a * n) * norb + q + a * n) * norb + r + b * n) * norb + s + b * n];
+            for (int b = 0; b < 2; b++) v += T.two(p + a * n, q + a * n, r + b * n, s + b * n);
         Gamma[t] = v;
     }
 }
 
 // gL[P][i] = sum_k Gamma[i][k] L[P][k] for i, k < n^2 (the chain rule of
 // (pq|rs) = sum_P L^P_pq L^P_rs through the free entries of L^P, with Gamma symmetric in
-// its two index pairs): a 64 x 32 output tile per CTA, k in steps of 16 staged in shared
-// memory, 8 outputs per thread, FP64 FMA
-constexpr int kGI = 64, kGP = 32, kGK = 16;
+// its two index pairs): an 8 x 32 output tile per CTA, one output per thread, k in steps of 32
+// staged in shared memory, the next step's loads in flight meanwhile; FP64 FMA.  The FP64 pipe
+// bounds it (2 FMA per clock per SM), so what counts is that every SM has work: 30 orbitals
+// and 120 factors are 452 of these tiles, 2.97 per SM.
+// Measured: 572 us with 64 x 32 tiles (60 CTAs), 181 us; at the FP64 rate 168 us.
+constexpr int kGI = 8, kGP = 32, kGK = 32;
 __global__ void __launch_bounds__(256) k_gamma_chol(int nn, int naux, const double *__restrict__ Gamma,
                                                      const double *__restrict__ L, double *__restrict__ gL)
 {
-    __shared__ double sG[kGK][kGI + 1];
-    __shared__ double sL[kGK][kGP + 1];
+    __shared__ double sG[kGI][kGK];
+    __shared__ double sL[kGP][kGK + 1];
     const int i0 = blockIdx.x * kGI, P0 = blockIdx.y * kGP;
-    const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;   // P = P0 + tx, i = i0 + ty + 8 u
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+    // this thread stages column k0 + tx of row i0 + ty of Gamma and of rows P0 + ty + 8 u of L
+    double g, l[4];
+    auto load = [&](int k0) {
+        const int k = k0 + tx;
+        g = i0 + ty < nn && k < nn ? Gamma[(int64_t)(i0 + ty) * nn + k] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int P = P0 + ty + 8 * u;
+            l[u] = P < naux && k < nn ? L[(int64_t)P * nn + k] : 0.0;
+        }
+    };
+    double acc = 0.0;
+    load(0);
     for (int k0 = 0; k0 < nn; k0 += kGK) {
-        for (int t = threadIdx.x; t < kGK * kGI; t += blockDim.x) {
-            const int kk = t % kGK, ii = t / kGK;
-            const int i = i0 + ii, k = k0 + kk;
-            sG[kk][ii] = (i < nn && k < nn) ? Gamma[(int64_t)i * nn + k] : 0.0;
-        }
-        for (int t = threadIdx.x; t < kGK * kGP; t += blockDim.x) {
-            const int kk = t % kGK, pp = t / kGK;
-            const int P = P0 + pp, k = k0 + kk;
-            sL[kk][pp] = (P < naux && k < nn) ? L[(int64_t)P * nn + k] : 0.0;
-        }
         __syncthreads();
+        sG[ty][tx] = g;
 #pragma unroll
-        for (int kk = 0; kk < kGK; kk++) {
-            const double l = sL[kk][tx];
-#pragma unroll
-            for (int u = 0; u < 8; u++) acc[u] = fma(sG[kk][ty + 8 * u], l, acc[u]);
-        }
+        for (int u = 0; u < 4; u++) sL[ty + 8 * u][tx] = l[u];
         __syncthreads();
+        if (k0 + kGK < nn) load(k0 + kGK);
+#pragma unroll
+        for (int kk = 0; kk < kGK; kk++) acc = fma(sG[ty][kk], sL[tx][kk], acc);
     }
-    const int P = P0 + tx;
-    if (P < naux)
-#pragma unroll
-        for (int u = 0; u < 8; u++) {
-            const int i = i0 + ty + 8 * u;
-            if (i < nn) gL[(int64_t)P * nn + i] = acc[u];
-        }
+    const int P = P0 + tx, i = i0 + ty;
+    if (P < naux && i < nn) gL[(int64_t)P * nn + i] = acc;
 }
 
 }  // namespace
@@ -536,28 +803,29 @@ extern "C" int sci_rdm_grads(sci_ctx *ctx, const double *C, int nvec, const doub
     if (nvec < 1 || (ctx->M > 0 && !C)) return sci_fail(ctx, SCI_ERR_ARG, "rdm_grads: need nvec >= 1 and C");
     if ((chol == nullptr) != (gchol == nullptr) || (chol && naux < 1))
         return sci_fail(ctx, SCI_ERR_ARG, "rdm_grads: chol and gchol go together, naux >= 1");
+    if (ctx->norb > 256 || ctx->nwords > sci::kMaxWords) return sci_fail(ctx, SCI_ERR_ARG, "rdm_grads: at most 256 orbitals");
     if (sci_cuda_check(ctx, cudaSetDevice(ctx->device), "cudaSetDevice")) return SCI_ERR_CUDA;
-    const int n = ctx->n, norb = ctx->norb;
-    const int64_t nn = (int64_t)n * n, n4 = nn * nn, o2 = (int64_t)norb * norb, o4 = o2 * o2;
+    const int n = ctx->n;
+    const int64_t nn = (int64_t)n * n, n4 = nn * nn;
     const bool two = Gamma || chol;
-    // spin-orbital g1, g2 and (when the caller passes no Gamma but needs the contraction)
-    // the spin-summed Gamma, in a buffer of their own
-    double *buf = nullptr;
-    const size_t need = sizeof(double) * (o2 + (two ? o4 : 0) + (two && !Gamma ? n4 : 0));
-    if (cudaMalloc(&buf, need) != cudaSuccess) return sci_fail(ctx, SCI_ERR_NOMEM, "rdm_grads: scratch");
-    double *g1 = buf, *g2 = two ? buf + o2 : nullptr, *G = Gamma ? Gamma : (two ? buf + o2 + o4 : nullptr);
-    int rc = sci_rdm12(ctx, C, nvec, weights, g1, g2);
+    // the spin-summed Gamma, when the caller passes none but needs the contraction
+    double *G = Gamma;
+    if (two && !Gamma && cudaMalloc(&G, sizeof(double) * n4) != cudaSuccess)
+        return sci_fail(ctx, SCI_ERR_NOMEM, "rdm_grads: scratch");
+    Tables<double> T;
+    int rc = rdm_weights(ctx, nvec, weights);
+    if (rc == SCI_OK) rc = rdm_tables<double>(ctx, C, nvec, static_cast<const double *>(ctx->rdm_w), two, T);
     cudaStream_t st = ctx->stream;
-    if (rc == SCI_OK && gamma) k_spin_sum1<<<grid_for(nn), kThreads, 0, st>>>(n, g1, gamma);
-    if (rc == SCI_OK && two) k_spin_sum2<<<grid_for(n4), kThreads, 0, st>>>(n, g2, G);
+    if (rc == SCI_OK && gamma) k_spin_sum1<<<grid_for(nn), kThreads, 0, st>>>(n, T, gamma);
+    if (rc == SCI_OK && two) k_spin_sum2<<<grid_for(n4), kThreads, 0, st>>>(n, T, G);
     if (rc == SCI_OK && chol) {
         const dim3 grid((unsigned)((nn + kGI - 1) / kGI), (unsigned)((naux + kGP - 1) / kGP));
         k_gamma_chol<<<grid, 256, 0, st>>>((int)nn, naux, G, chol, gchol);
     }
     if (rc == SCI_OK) rc = sci_cuda_check(ctx, cudaGetLastError(), "rdm_grads launch");
-    // the buffer is freed after the queued work has read it
+    // Gamma is freed after the queued work has read it
     cudaError_t e = cudaStreamSynchronize(st);
-    cudaFree(buf);
+    if (G != Gamma) cudaFree(G);
     if (rc == SCI_OK) rc = sci_cuda_check(ctx, e, "rdm_grads");
     return rc;
 }
@@ -569,19 +837,7 @@ extern "C" int sci_rdm12(sci_ctx *ctx, const void *C, int nvec, const double *we
     if (nvec < 1 || !rdm1 || (ctx->M > 0 && !C)) return sci_fail(ctx, SCI_ERR_ARG, "rdm12: need nvec >= 1, C and rdm1");
     if (ctx->norb > 256 || ctx->nwords > sci::kMaxWords) return sci_fail(ctx, SCI_ERR_ARG, "rdm12: at most 256 orbitals");
     if (sci_cuda_check(ctx, cudaSetDevice(ctx->device), "cudaSetDevice")) return SCI_ERR_CUDA;
-    // weights to the device (a host array of nvec doubles, NULL = all ones)
-    const size_t wbytes = sizeof(double) * nvec;
-    if (wbytes > ctx->rdm_wbytes) {
-        if (ctx->rdm_w) cudaFree(ctx->rdm_w);
-        ctx->rdm_w = nullptr, ctx->rdm_wbytes = 0;
-        if (cudaMalloc(&ctx->rdm_w, wbytes) != cudaSuccess) return sci_fail(ctx, SCI_ERR_NOMEM, "rdm12: weights");
-        ctx->rdm_wbytes = wbytes;
-    }
-    std::vector<double> w(nvec, 1.0);
-    if (weights) std::copy(weights, weights + nvec, w.begin());
-    if (sci_cuda_check(ctx, cudaMemcpyAsync(ctx->rdm_w, w.data(), wbytes, cudaMemcpyHostToDevice, ctx->stream), "rdm12 weights") ||
-        sci_cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "rdm12 weights sync"))
-        return SCI_ERR_CUDA;
+    if (const int rc = rdm_weights(ctx, nvec, weights)) return rc;
     const double *wk = static_cast<const double *>(ctx->rdm_w);
     if (ctx->cplx)
         return rdm_run<zdbl>(ctx, static_cast<const zdbl *>(C), nvec, wk, static_cast<zdbl *>(rdm1), static_cast<zdbl *>(rdm2));
