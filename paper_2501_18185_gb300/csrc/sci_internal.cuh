@@ -170,6 +170,7 @@ struct sci_ctx {
     void *h_so = nullptr;   // [norb][norb], spin-orbital h (scalar)
     void *jd = nullptr;     // [norb][norb] (ii|jj)
     void *kd = nullptr;     // [norb][norb] (ij|ji)
+    double *gd = nullptr;   // [norb][norb] Re (ii|jj) - Re (ij|ji)
     void *g_so = nullptr;   // [norb][norb][norb]
     void *tab = nullptr;    // pair table (scalar)
     float *tab32 = nullptr; // FP32 copy of tab (real mode)
