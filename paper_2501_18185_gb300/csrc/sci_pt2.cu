@@ -54,7 +54,6 @@
 #include <vector>
 
 #include "sci_bits.cuh"
-#include "sci_ds.cuh"
 #include "sci_internal.cuh"
 
 namespace {
@@ -69,8 +68,9 @@ struct Pt2 {
     int n, norb, na, nb;
     uint64_t ref, ref_hi, ref_w2;   // the reference string: orbitals 0..63, 64..127, 128..191
     const double *tab, *fref, *g_so;
-    const double *fdiag, *G;  // [norb], [norb][norb]
     const double *Eref;
+    const double *fix_scale;  // F and G as integers in units of 1 / fix_scale: [norb], [norb][norb]
+    const long long *fix;
     uint32_t gcode[192];      // codes of the beta orbitals (spin-orbital mode) or spinors
     uint8_t obc[192];         // those orbitals sorted by code
     uint8_t cstart[(1 << kMaxBits) + 1];  // first index in obc of each code
@@ -316,6 +316,36 @@ __device__ __forceinline__ void insert(const Pt2 &p, K I, double hij, const doub
     for (int v = 0; v < R; v++) atomicAdd(reinterpret_cast<double *>(slot + KW + v), hij * cJ[v]);
 }
 
+// The same by a whole warp, each lane with an excitation of the warp's J when `ok`.  The L2's
+// rate of random requests bounds the generation (about 5e10 a second over keys, claims and
+// adds), and the lanes of one instruction that add to one 32-byte sector are one request.  So G
+// lanes (R rounded up to a power of two) take a slot, one root each: cs is the coefficient of
+// this lane's root, lane % G.  Generation of 24 orbitals, M = 40k: two roots 41.9 -> 33.0 ms, four
+// 66.7 -> 48.7; one root is unchanged.  (Tables that fit the L2, W split into more parts, were
+// slower: 53.8 ms at 128 MB, two roots.)
+template <int R> __device__ constexpr int coop_lanes() { return R == 1 ? 1 : R == 2 ? 2 : R <= 4 ? 4 : 8; }
+template <int R, int KW, typename K>
+__device__ __forceinline__ void insert_warp(const Pt2 &p, bool ok, K I, double hij, double cs, double cmax, uint32_t &nc,
+                                            int lane)
+{
+    constexpr int G = coop_lanes<R>();
+    if (ok && p.eps > 0.0 && fabs(hij) * cmax < p.eps) ok = false;
+    uint64_t *slot = ok ? claim<KW, R>(p, I, nc) : nullptr;
+    __syncwarp();
+    if constexpr (G == 1) {
+        if (slot) atomicAdd(reinterpret_cast<double *>(slot + KW), hij * cs);
+    } else {
+        const int sub = lane % G;
+#pragma unroll
+        for (int r = 0; r < G; r++) {
+            const int src = r * (32 / G) + lane / G;
+            const unsigned long long a = __shfl_sync(0xffffffffu, (unsigned long long)slot, src);
+            const double h = __shfl_sync(0xffffffffu, hij, src);
+            if (a && sub < R) atomicAdd(reinterpret_cast<double *>(a) + KW + sub, h * cs);
+        }
+    }
+}
+
 // The alpha (bits 0..n-1) and beta (bits n..2n-1) strings of a spin-orbital key.  One-
 // and two-word keys give 32- or 64-bit strings (n <= 64); three-word keys (n <= 96) give
 // two-word strings.
@@ -454,6 +484,7 @@ k_pt2_gen(const uint64_t *__restrict__ Pkeys, int64_t M, const double *__restric
         double cJ[R], cmax = 0.0;
 #pragma unroll
         for (int v = 0; v < R; v++) cJ[v] = C[J * R + v], cmax = fmax(cmax, fabs(cJ[v]));
+        const double cs = C[J * R + min(lane % coop_lanes<R>(), R - 1)];   // of insert_warp()
         __syncwarp();
         for (int o = lane; o < n; o += 32) {
             if constexpr (KW == 3) {
@@ -478,18 +509,26 @@ k_pt2_gen(const uint64_t *__restrict__ Pkeys, int64_t M, const double *__restric
         // alpha singles and alpha-alpha doubles: the beta string is unchanged
         if (target == 0) {
             const int c0 = na * ua, qa = ua * (ua - 1) / 2, c2 = na * (na - 1) / 2 * qa;
-            for (int t = lane; t < c0 + c2; t += 32) {
-                if (t < c0) {
-                    const int i = orb[t / ua], a = orb[NO + t % ua];
-                    insert<R, KW>(p, (key & ~bitk<K>(i)) | bitk<K>(a), h_single(p, key, i, a), cJ, cmax, nclaim);
-                } else {
-                    const int s = t - c0;
+            for (int t = lane; t < c0; t += 32) {
+                const int i = orb[t / ua], a = orb[NO + t % ua];
+                insert<R, KW>(p, (key & ~bitk<K>(i)) | bitk<K>(a), h_single(p, key, i, a), cJ, cmax, nclaim);
+            }
+            __syncwarp();
+            for (int base = 0; base < c2; base += 32) {
+                const int s = base + lane;
+                bool ok = s < c2;
+                K I{};
+                double h = 0.0;
+                if (ok) {
                     const uint16_t po = pair_of(s / qa), pv = pair_of(s % qa);
                     const int i = orb[po & 0xFF], j = orb[po >> 8], a = orb[NO + (pv & 0xFF)], b = orb[NO + (pv >> 8)];
-                    if (p.bss && p.bss[j * (j - 1) / 2 + i] * cmax < p.eps) continue;   // the class's bound
-                    const K I = (key & ~bitk<K>(i) & ~bitk<K>(j)) | bitk<K>(a) | bitk<K>(b);
-                    insert<R, KW>(p, I, h_double(p, key, i, j, a, b), cJ, cmax, nclaim);
+                    ok = !(p.bss && p.bss[j * (j - 1) / 2 + i] * cmax < p.eps);   // the class's bound
+                    if (ok) {
+                        I = (key & ~bitk<K>(i) & ~bitk<K>(j)) | bitk<K>(a) | bitk<K>(b);
+                        h = h_double(p, key, i, j, a, b);
+                    }
                 }
+                insert_warp<R, KW>(p, ok, I, h, cs, cmax, nclaim, lane);
             }
         }
 
@@ -509,18 +548,27 @@ k_pt2_gen(const uint64_t *__restrict__ Pkeys, int64_t M, const double *__restric
         }
         __syncwarp();
         const int nl = s_nl[w], c0 = na * ua;
-        for (int t = lane; t < nl * (1 + c0); t += 32) {
-            const uint16_t e = s_list[w][t / (1 + c0)];
-            const int jb = n + (e & 0xFF), vb_ = n + (e >> 8);
-            const int s = t % (1 + c0);
-            if (s == 0) {
-                insert<R, KW>(p, (key & ~bitk<K>(jb)) | bitk<K>(vb_), h_single(p, key, jb, vb_), cJ, cmax, nclaim);
-            } else {
-                const int i = orb[(s - 1) / ua], a = orb[NO + (s - 1) % ua];
-                if (p.bab && p.bab[(e & 0xFF) * n + i] * cmax < p.eps) continue;   // the class's bound
-                const K I = (key & ~bitk<K>(i) & ~bitk<K>(jb)) | bitk<K>(a) | bitk<K>(vb_);
-                insert<R, KW>(p, I, h_double(p, key, i, jb, a, vb_), cJ, cmax, nclaim);
+        for (int t = lane; t < nl; t += 32) {
+            const int jb = n + (s_list[w][t] & 0xFF), vb_ = n + (s_list[w][t] >> 8);
+            insert<R, KW>(p, (key & ~bitk<K>(jb)) | bitk<K>(vb_), h_single(p, key, jb, vb_), cJ, cmax, nclaim);
+        }
+        __syncwarp();
+        for (int base = 0; base < nl * c0; base += 32) {
+            const int t = base + lane;
+            bool ok = t < nl * c0;
+            K I{};
+            double h = 0.0;
+            if (ok) {
+                const uint16_t e = s_list[w][t / c0];
+                const int jb = n + (e & 0xFF), vb_ = n + (e >> 8), s = t % c0;
+                const int i = orb[s / ua], a = orb[NO + s % ua];
+                ok = !(p.bab && p.bab[(e & 0xFF) * n + i] * cmax < p.eps);   // the class's bound
+                if (ok) {
+                    I = (key & ~bitk<K>(i) & ~bitk<K>(jb)) | bitk<K>(a) | bitk<K>(vb_);
+                    h = h_double(p, key, i, jb, a, vb_);
+                }
             }
+            insert_warp<R, KW>(p, ok, I, h, cs, cmax, nclaim, lane);
         }
 
         // beta-beta doubles j1 < j2 -> b1 < b2: for each occupied pair and first virtual
@@ -698,11 +746,16 @@ k_pt2_gen_z(const uint64_t *__restrict__ Pkeys, int64_t M, const zdbl *__restric
 }
 
 // sum over the table entries of num^2 / (E0 - H_II).  Each warp packs the occupied slots
-// it scans into a buffer of 32 and evaluates full buffers, so every lane works; H_II
-// (E_ref plus O(level^2) table terms) is summed in paired FP32 from split copies of F and
-// G in shared memory, and added to E_ref in FP64.
-// GS: G in shared memory (up to 168 orbitals); else read from global memory and split on
-// the fly.
+// it scans into a buffer of 32 and evaluates full buffers, so every lane works.  Instruction
+// issue bounds it, so H_II - E_ref (O(level^2) table terms) is summed as 64-bit integers: F and
+// G in units of 1 / fix_scale, chosen by k_pt2_setup so that no sum overflows (exact sums of
+// terms rounded to 2^-62 of their largest total, two integer adds a term), and the inner
+// loops run over a list of the differing orbitals in shared memory, not over bits.
+// Against paired-FP32 sums over bits: 30 orbitals, M = 60k, one root, 2.4e8 determinants 20.4 ->
+// 13.2 ms; 24 orbitals, M = 40k, two roots, 1.4e8 determinants 13.5 -> 12.5 (the FP64 divisions,
+// one a root, bind there).
+// GS: G in shared memory (up to 162 orbitals); else read from global memory.
+constexpr int kDiffList = 32;   // orbitals of the list; determinants that differ in more walk bits
 template <int R, bool CPLX, int KW, bool GS = true>
 __global__ void __launch_bounds__(kThreads)
 k_pt2_eval(Pt2 p, uint64_t cap, const double *__restrict__ E0, double *__restrict__ out)
@@ -710,19 +763,19 @@ k_pt2_eval(Pt2 p, uint64_t cap, const double *__restrict__ E0, double *__restric
     using K = typename KeyOf<KW>::T;
     constexpr int NW = CPLX ? 2 * R : R;   // value words per slot
     constexpr int SW = slot_words<KW, NW>();
-    extern __shared__ float2 s_gf[];       // F [norb], then G [norb][norb] (dynamic)
+    extern __shared__ long long s_gf[];    // F [norb], then G [norb][norb] (dynamic)
     __shared__ uint64_t sbuf[kWarps][64];
     __shared__ double red[kWarps][R];
+    __shared__ uint8_t s_diff[kDiffList][kThreads];
     const int norb = p.norb;
-    float2 *sF = s_gf, *sGs = s_gf + norb;
-    for (int t = threadIdx.x; t < norb; t += blockDim.x) sF[t] = sci::ds_split_int(p.fdiag[t]);
-    if constexpr (GS)
-        for (int t = threadIdx.x; t < norb * norb; t += blockDim.x) sGs[t] = sci::ds_split_int(p.G[t]);
+    const long long *sF = s_gf, *sGs = s_gf + norb;
+    for (int t = threadIdx.x; t < norb * (GS ? norb + 1 : 1); t += blockDim.x) s_gf[t] = p.fix[t];
     __syncthreads();
-    auto gget = [&](int t) -> float2 {
+    auto gget = [&](int t) -> long long {
         if constexpr (GS) return sGs[t];
-        else return sci::ds_split_int(__ldg(p.G + t));
+        else return __ldg(p.fix + norb + t);
     };
+    const double unit = 1.0 / *p.fix_scale;
     const double Eref = *p.Eref;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     double acc[R], e0[R];
@@ -736,24 +789,40 @@ k_pt2_eval(Pt2 p, uint64_t cap, const double *__restrict__ E0, double *__restric
         else if constexpr (KW == 2) I = W2(slot[0], slot[1]);
         else I = W3(slot[0], slot[1], ~slot[2]);
         const K H = ref & ~I, Pm = I & ~ref;
-        sci::Ds e;
-        sci::ds_zero(e);
-        for (K m = H; m; m &= m - 1) {
-            const int i = lowbit(m);
-            const float2 f = sF[i];
-            sci::ds_add(e, make_float2(-f.x, -f.y));
-            for (K m2 = m & (m - 1); m2; m2 &= m2 - 1) sci::ds_add(e, gget(i * norb + lowbit(m2)));
-            for (K m2 = Pm; m2; m2 &= m2 - 1) {
-                const float2 g = gget(i * norb + lowbit(m2));
-                sci::ds_add(e, make_float2(-g.x, -g.y));
+        long long e = 0;
+        if (popck(H) + popck(Pm) <= kDiffList) {
+            uint8_t *list = &s_diff[0][threadIdx.x];
+            int nh = 0, nd = 0;
+            for (K m = H; m; m &= m - 1, nh++) {
+                const int i = lowbit(m), gi = i * norb;
+                e -= sF[i];
+                for (int k = 0; k < nh; k++) e += gget(gi + list[k * kThreads]);
+                list[nh * kThreads] = (uint8_t)i;
+            }
+            nd = nh;
+            for (K m = Pm; m; m &= m - 1, nd++) {
+                const int a = lowbit(m), ga = a * norb;
+                long long minus = 0;
+                e += sF[a];
+                for (int k = 0; k < nh; k++) minus += gget(ga + list[k * kThreads]);
+                for (int k = nh; k < nd; k++) e += gget(ga + list[k * kThreads]);
+                e -= minus;
+                list[nd * kThreads] = (uint8_t)a;
+            }
+        } else {
+            for (K m = H; m; m &= m - 1) {
+                const int i = lowbit(m);
+                e -= sF[i];
+                for (K m2 = m & (m - 1); m2; m2 &= m2 - 1) e += gget(i * norb + lowbit(m2));
+                for (K m2 = Pm; m2; m2 &= m2 - 1) e -= gget(i * norb + lowbit(m2));
+            }
+            for (K m = Pm; m; m &= m - 1) {
+                const int a = lowbit(m);
+                e += sF[a];
+                for (K m2 = m & (m - 1); m2; m2 &= m2 - 1) e += gget(a * norb + lowbit(m2));
             }
         }
-        for (K m = Pm; m; m &= m - 1) {
-            const int a = lowbit(m);
-            sci::ds_add(e, sF[a]);
-            for (K m2 = m & (m - 1); m2; m2 &= m2 - 1) sci::ds_add(e, gget(a * norb + lowbit(m2)));
-        }
-        const double hii = Eref + sci::ds_value(e);
+        const double hii = Eref + (double)e * unit;
 #pragma unroll
         for (int v = 0; v < R; v++) {
             double num2;
@@ -849,19 +918,35 @@ __device__ __forceinline__ double re_of(zdbl a) { return a.x; }
 template <typename T>
 __global__ void k_pt2_setup(int norb, uint64_t ref_lo, uint64_t ref_hi, uint64_t ref_w2, const T *__restrict__ h_so,
                             const T *__restrict__ jd, const T *__restrict__ kd, double *__restrict__ G,
-                            double *__restrict__ fdiag, double *__restrict__ Eref)
+                            double *__restrict__ fdiag, double *__restrict__ Eref, double *__restrict__ fix_scale,
+                            long long *__restrict__ fix)
 {
+    __shared__ unsigned long long s_max[2];   // largest |F| and |G|, as bits (ordered like the values)
+    if (threadIdx.x < 2) s_max[threadIdx.x] = 0ull;
     const W3 ref(ref_lo, ref_hi, ref_w2);
     for (int t = threadIdx.x; t < norb * norb; t += blockDim.x) {
         const int a = t / norb, b = t % norb;
         G[t] = a == b ? 0.0 : re_of(jd[t]) - re_of(kd[t]);
     }
     __syncthreads();
+    for (int t = threadIdx.x; t < norb * norb; t += blockDim.x)
+        atomicMax(&s_max[1], (unsigned long long)__double_as_longlong(fabs(G[t])));
     for (int a = threadIdx.x; a < norb; a += blockDim.x) {
         double f = re_of(h_so[a * norb + a]);
         for (W3 m = ref; m; m &= m - 1) f += G[a * norb + lowbit(m)];
         fdiag[a] = f;
+        atomicMax(&s_max[0], (unsigned long long)__double_as_longlong(fabs(f)));
     }
+    __syncthreads();
+    // F and G as integers: the largest power of two that keeps any sum of them below 2^62
+    const double bound = norb * __longlong_as_double((long long)s_max[0]) +
+                         0.5 * norb * norb * __longlong_as_double((long long)s_max[1]);
+    int ex = 0;
+    frexp(bound, &ex);   // bound < 2^ex
+    const double scale = ldexp(1.0, min(62 - ex, 1000));
+    if (threadIdx.x == 0) *fix_scale = scale;
+    for (int t = threadIdx.x; t < norb; t += blockDim.x) fix[t] = llrint(fdiag[t] * scale);
+    for (int t = threadIdx.x; t < norb * norb; t += blockDim.x) fix[norb + t] = llrint(G[t] * scale);
     if (threadIdx.x == 0) {
         double e = 0.0;
         for (W3 m = ref; m; m &= m - 1) {
@@ -940,7 +1025,7 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
         if (tab2) cudaFree(tab2);
         if (bnd_free) cudaFree(bnd_free);
     };
-    const size_t nsmall = (size_t)R * 3 + (size_t)norb * norb + norb + 1 + 2;
+    const size_t nsmall = (size_t)R * 3 + 2 * ((size_t)norb * norb + norb) + 2 + 2;
     if (cudaMalloc(&S, sizeof(double) * SC * std::max<int64_t>(1, M) * R) != cudaSuccess ||
         cudaMalloc(&small, sizeof(double) * nsmall) != cudaSuccess) {
         cleanup();
@@ -948,7 +1033,9 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
     }
     double *dE0 = small, *outW = small + R, *outP = small + 2 * R, *G = small + 3 * R, *fdiag = G + norb * norb,
            *Eref = fdiag + norb;
-    unsigned long long *count = reinterpret_cast<unsigned long long *>(Eref + 1);
+    double *fix_scale = Eref + 1;
+    long long *fix = reinterpret_cast<long long *>(fix_scale + 1);
+    unsigned long long *count = reinterpret_cast<unsigned long long *>(fix + norb * norb + norb);
     int *flag = reinterpret_cast<int *>(count + 1);
     if (sci_cuda_check(ctx, cudaMemsetAsync(small, 0, sizeof(double) * nsmall, st), "enpt2 memset") ||
         sci_cuda_check(ctx, cudaMemcpyAsync(dE0, E0h, sizeof(double) * R, cudaMemcpyHostToDevice, st), "enpt2 E0")) {
@@ -970,10 +1057,10 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
     }
     if constexpr (SPIN)
         k_pt2_setup<zdbl><<<1, 256, 0, st>>>(norb, ctx->ref, ctx->ref_hi, ctx->ref_w2, (const zdbl *)ctx->h_so,
-                                             (const zdbl *)ctx->jd, (const zdbl *)ctx->kd, G, fdiag, Eref);
+                                             (const zdbl *)ctx->jd, (const zdbl *)ctx->kd, G, fdiag, Eref, fix_scale, fix);
     else
         k_pt2_setup<double><<<1, 256, 0, st>>>(norb, ctx->ref, ctx->ref_hi, ctx->ref_w2, (const double *)ctx->h_so,
-                                               (const double *)ctx->jd, (const double *)ctx->kd, G, fdiag, Eref);
+                                               (const double *)ctx->jd, (const double *)ctx->kd, G, fdiag, Eref, fix_scale, fix);
     // the table: capacity a power of two within the budget
     const size_t slot = sizeof(uint64_t) * SW;
     uint64_t cap = 1ull << 8;  // at least 256 entries
@@ -1022,7 +1109,7 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
     }
     p.n = n, p.norb = norb, p.na = na, p.nb = nb, p.ref = ctx->ref, p.ref_hi = ctx->ref_hi, p.ref_w2 = ctx->ref_w2;
     p.tab = (const double *)ctx->tab, p.fref = (const double *)ctx->fref, p.g_so = (const double *)ctx->g_so;
-    p.fdiag = fdiag, p.G = G, p.Eref = Eref;
+    p.Eref = Eref, p.fix_scale = fix_scale, p.fix = fix;
     p.tab2 = tab2, p.mask = cap - 1, p.count = count, p.flag = flag;
     p.limit = (unsigned long long)(0.85 * (double)cap);
     p.eps = eps;
@@ -1052,13 +1139,13 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
         std::vector<int> fill(cnt.begin(), cnt.end() - 1);
         for (int o = 0; o < n; o++) p.obc[fill[p.gcode[o]]++] = (uint8_t)o;
     };
-    // the evaluation kernel's F and G (paired floats) in dynamic shared memory; past 165
+    // the evaluation kernel's F and G (integers) in dynamic shared memory; past 162
     // orbitals (three-word keys only) G is read from global memory
-    size_t eval_smem = sizeof(float2) * ((size_t)norb * norb + norb);
-    const bool eval_gs = KW < 3 || eval_smem <= 216 * 1024;
+    size_t eval_smem = sizeof(long long) * ((size_t)norb * norb + norb);
+    const bool eval_gs = KW < 3 || eval_smem <= 208 * 1024;
     auto keval = k_pt2_eval<R, SPIN, KW, true>;
     if constexpr (KW == 3)
-        if (!eval_gs) keval = k_pt2_eval<R, SPIN, KW, false>, eval_smem = sizeof(float2) * norb;
+        if (!eval_gs) keval = k_pt2_eval<R, SPIN, KW, false>, eval_smem = sizeof(long long) * norb;
     if (sci_cuda_check(ctx, cudaFuncSetAttribute(keval, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eval_smem),
                        "enpt2 eval attr"))
         return done(SCI_ERR_CUDA);
