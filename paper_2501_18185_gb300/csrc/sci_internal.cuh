@@ -21,9 +21,7 @@
 //       e2_idx[p]     determinant index of the member
 //       e2_code[p]    bits 0-7 x, bits 8-15 y: the two extra orbitals x < y of the
 //                     member (D = K | 2^x | 2^y); bit 16 the phase parity
-//                     #(K below x) + #(K below y); bits 17-22 the member's position
-//                     inside its y-group (members of the bucket with the same y);
-//                     bits 23-29 the y-group size
+//                     #(K below x) + #(K below y)
 //       e2_pos[p]     bits 0-15 position inside the bucket, bits 16-31 bucket size
 //     Table offsets are derived from (x, y) by pair_offsets().
 //   Singles table "B1": the same with (N-1)-electron keys S = D minus one bit.
@@ -55,11 +53,9 @@ enum DevErr : int {
 __host__ __device__ __forceinline__ int code_x(uint32_t c) { return (int)(c & 0xFFu); }
 __host__ __device__ __forceinline__ int code_y(uint32_t c) { return (int)((c >> 8) & 0xFFu); }
 __host__ __device__ __forceinline__ bool code_par(uint32_t c) { return (c >> 16) & 1u; }
-__host__ __device__ __forceinline__ int code_gofs(uint32_t c) { return (int)((c >> 17) & 0x3Fu); }
-__host__ __device__ __forceinline__ int code_gsize(uint32_t c) { return (int)((c >> 23) & 0x7Fu); }
-__host__ __device__ __forceinline__ uint32_t make_code(int x, int y, int par, int gofs, int gsize)
+__host__ __device__ __forceinline__ uint32_t make_code(int x, int y, int par)
 {
-    return (uint32_t)x | ((uint32_t)y << 8) | ((uint32_t)par << 16) | ((uint32_t)gofs << 17) | ((uint32_t)gsize << 23);
+    return (uint32_t)x | ((uint32_t)y << 8) | ((uint32_t)par << 16);
 }
 __host__ __device__ __forceinline__ int pos_off(uint32_t p) { return (int)(p & 0xFFFFu); }
 __host__ __device__ __forceinline__ int pos_size(uint32_t p) { return (int)(p >> 16); }

@@ -304,7 +304,7 @@ __global__ void k_validate(const uint64_t *__restrict__ keys, int64_t M, KeyRule
 
 // H_II = sum_{i in occ} h_ii + sum_{i<j in occ} [(ii|jj) - (ij|ji)].  Bound by the FP64 adds:
 // one per pair of electrons, with the differences tabulated (gd).
-// 30 orbitals, 20 electrons, M = 400k: 431 us with both orders of a pair and two table reads
+// 30 orbitals, 20 electrons, M = 250k: 431 us with both orders of a pair and two table reads
 // each, 113 us.
 template <typename S, int KW>
 __global__ void k_diag(const uint64_t *__restrict__ keys, int64_t M, int norb, const S *__restrict__ h_so,
@@ -341,7 +341,43 @@ __global__ void k_fref(int norb, Kw<sci::kMaxWords> ref, const S *__restrict__ h
     fref[t] = f;
 }
 
-// every determinant emits its keys with `holes` occupied bits removed (1 or 2): the key
+// One-word keys: every determinant emits its keys with `holes` occupied bits removed and its
+// index (the removed bits are those of the determinant outside the key).  A warp takes a
+// determinant, its lanes the pairs of its orbitals, so that the stores, 12 bytes an entry,
+// are consecutive and bound it; the order within a determinant is free, its keys all differ.
+// With a 4-byte index in place of an 8-byte value the sort moves a quarter less and its buffers
+// are smaller; loading 400k determinants of 30 orbitals took 22.0 ms with a thread per
+// determinant and 8-byte values, 15.0 now.
+__global__ void __launch_bounds__(256) k_emit1(const uint64_t *__restrict__ keys, int64_t M, int holes, int per_det,
+                                               uint64_t *__restrict__ out, uint32_t *__restrict__ out_idx)
+{
+    __shared__ uint8_t s_orb[8][64];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint8_t *orb = s_orb[wid];
+    for (int64_t I = blockIdx.x * (int64_t)8 + wid; I < M; I += (int64_t)gridDim.x * 8) {
+        const uint64_t k = keys[I];
+        __syncwarp();
+        for (int o = lane; o < 64; o += 32)
+            if ((k >> o) & 1) orb[__popcll(k & ((1ull << o) - 1))] = (uint8_t)o;
+        __syncwarp();
+        const int64_t base = I * per_det;
+        for (int t = lane; t < per_det; t += 32) {
+            uint64_t e = k;
+            if (holes == 1) {
+                e ^= 1ull << orb[t];
+            } else {   // t = b(b-1)/2 + a, a < b
+                int b = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)t)) * 0.5f);
+                while (b * (b - 1) / 2 > t) b--;
+                while ((b + 1) * b / 2 <= t) b++;
+                e ^= 1ull << orb[b] | 1ull << orb[t - b * (b - 1) / 2];
+            }
+            out[base + t] = e;
+            out_idx[base + t] = (uint32_t)I;
+        }
+    }
+}
+
+// Keys of several words: every determinant emits its keys with `holes` occupied bits removed: the key
 // words (word w at out_w + w * stride) and the value I | x << 32 | y << 40
 template <int KW>
 __global__ void k_emit(const uint64_t *__restrict__ keys, int64_t M, int holes, int per_det, uint64_t *__restrict__ out_w,
@@ -410,13 +446,31 @@ __global__ void k_gather_sizes(const uint32_t *__restrict__ order, const uint32_
 
 
 
+// Sorted value `at` of the bucket of key K: the determinant, and its orbitals x (< y) outside K.
+// One-word lists sort 4-byte indices and read the orbitals off the determinant's key.
+template <int KW>
+__device__ __forceinline__ uint32_t member(const void *vals, const uint64_t *keys, const Kw<KW> &K, int64_t at, int &x,
+                                           int &y)
+{
+    if constexpr (KW == 1) {
+        const uint32_t I = static_cast<const uint32_t *>(vals)[at];
+        const uint64_t d = keys[I] ^ K.w[0];
+        x = __ffsll((long long)d) - 1, y = 63 - __clzll((long long)d);
+        return I;
+    } else {
+        const uint64_t v = static_cast<const uint64_t *>(vals)[at];
+        x = (int)((v >> 32) & 0xFF), y = (int)((v >> 40) & 0xFF);
+        return (uint32_t)v;
+    }
+}
+
 // warp per kept bucket: scatter members into the final doubles table.  Members of a
-// bucket arrive in ascending determinant order, i.e. ascending (y, x); a y-group is the
-// run of members with the same y.
+// bucket arrive in ascending determinant order, i.e. ascending (y, x).
 template <int KW>
 __global__ void k_fill2(const uint32_t *__restrict__ order, const uint32_t *__restrict__ counts,
                         const uint32_t *__restrict__ offsets, const uint32_t *__restrict__ newoff,
-                        const uint64_t *__restrict__ ukeys, const uint64_t *__restrict__ vals, int64_t kept,
+                        const uint64_t *__restrict__ ukeys, const void *__restrict__ vals,
+                        const uint64_t *__restrict__ keys, int64_t kept,
                         uint32_t *__restrict__ e_idx, uint32_t *__restrict__ e_code, uint32_t *__restrict__ e_pos)
 {
     int lane = threadIdx.x & 31;
@@ -427,15 +481,11 @@ __global__ void k_fill2(const uint32_t *__restrict__ order, const uint32_t *__re
         uint32_t size = counts[b], old = offsets[b], dst = newoff[j];
         const Kw<KW> K = load_kw<KW>(ukeys, b);
         for (uint32_t t = lane; t < size; t += 32) {
-            uint64_t v = vals[old + t];
-            int x = (int)((v >> 32) & 0xFF), y = (int)((v >> 40) & 0xFF);
-            uint32_t gs = t, ge = t + 1;
-            while (gs > 0 && (int)((vals[old + gs - 1] >> 40) & 0xFF) == y) gs--;
-            while (ge < size && (int)((vals[old + ge] >> 40) & 0xFF) == y) ge++;
-            int par = (below_w(K, x) + below_w(K, y)) & 1;
-            e_idx[dst + t] = (uint32_t)(v & 0xFFFFFFFFull);
-            // the y-group fields saturate (63, 127): no kernel reads them past that
-            e_code[dst + t] = sci::make_code(x, y, par, (int)min(t - gs, 63u), (int)min(ge - gs, 127u));
+            int x, y;
+            const uint32_t I = member<KW>(vals, keys, K, old + t, x, y);
+            const int par = (below_w(K, x) + below_w(K, y)) & 1;
+            e_idx[dst + t] = I;
+            e_code[dst + t] = sci::make_code(x, y, par);
             e_pos[dst + t] = t | (size << 16);
         }
     }
@@ -444,7 +494,8 @@ __global__ void k_fill2(const uint32_t *__restrict__ order, const uint32_t *__re
 template <int KW>
 __global__ void k_fill1(const uint32_t *__restrict__ order, const uint32_t *__restrict__ counts,
                         const uint32_t *__restrict__ offsets, const uint32_t *__restrict__ newoff,
-                        const uint64_t *__restrict__ ukeys, const uint64_t *__restrict__ vals, int64_t kept,
+                        const uint64_t *__restrict__ ukeys, const void *__restrict__ vals,
+                        const uint64_t *__restrict__ keys, int64_t kept,
                         uint32_t *__restrict__ e_idx, uint64_t *__restrict__ e_S, uint32_t *__restrict__ e_meta)
 {
     int lane = threadIdx.x & 31;
@@ -455,10 +506,10 @@ __global__ void k_fill1(const uint32_t *__restrict__ order, const uint32_t *__re
         uint32_t size = counts[b], old = offsets[b], dst = newoff[j];
         const Kw<KW> K = load_kw<KW>(ukeys, b);
         for (uint32_t t = lane; t < size; t += 32) {
-            uint64_t v = vals[old + t];
-            int x = (int)((v >> 32) & 0xFF);
+            int x, y;
+            const uint32_t I = member<KW>(vals, keys, K, old + t, x, y);
             uint32_t par = (uint32_t)(below_w(K, x) & 1);
-            e_idx[dst + t] = (uint32_t)(v & 0xFFFFFFFFull);
+            e_idx[dst + t] = I;
 #pragma unroll
             for (int w = 0; w < KW; w++) e_S[(int64_t)(dst + t) * KW + w] = K.w[w];
             e_meta[dst + t] = sci::make_meta(x, (int)par, (int)t, (int)size);
@@ -616,13 +667,12 @@ int build_buckets(sci_ctx *ctx, int holes, int per_det, Buckets &B)
     TmpBuf ka, kb, va;
     SCI_CK(cudaMalloc(&ka.p, total * 8));
     SCI_CK(cudaMalloc(&kb.p, total * 8));
-    SCI_CK(cudaMalloc(&va.p, total * 8));
-    SCI_CK(cudaMalloc(&B.vals_sorted.p, total * 8));
-    k_emit<1><<<grid_for(M), 256, 0, st>>>(ctx->keys, M, holes, per_det, ka.as<uint64_t>(), total,
-                                          va.as<uint64_t>());
+    SCI_CK(cudaMalloc(&va.p, total * 4));
+    SCI_CK(cudaMalloc(&B.vals_sorted.p, total * 4));
+    k_emit1<<<grid_for(M * 32), 256, 0, st>>>(ctx->keys, M, holes, per_det, ka.as<uint64_t>(), va.as<uint32_t>());
     SCI_CK(cudaGetLastError());
     cub::DoubleBuffer<uint64_t> dk(ka.as<uint64_t>(), kb.as<uint64_t>());
-    cub::DoubleBuffer<uint64_t> dv(va.as<uint64_t>(), B.vals_sorted.as<uint64_t>());
+    cub::DoubleBuffer<uint32_t> dv(va.as<uint32_t>(), B.vals_sorted.as<uint32_t>());
     int end_bit = ctx->norb;
     size_t tb = 0;
     SCI_CK(cub::DeviceRadixSort::SortPairs(nullptr, tb, dk, dv, nitems, 0, end_bit, st));
@@ -632,7 +682,7 @@ int build_buckets(sci_ctx *ctx, int holes, int per_det, Buckets &B)
         SCI_CK(cub::DeviceRadixSort::SortPairs(tmp.p, tb, dk, dv, nitems, 0, end_bit, st));
     }
     // keep the sorted values; release the other value buffer
-    if (dv.Current() != B.vals_sorted.as<uint64_t>()) std::swap(va.p, B.vals_sorted.p);
+    if (dv.Current() != B.vals_sorted.as<uint32_t>()) std::swap(va.p, B.vals_sorted.p);
     cudaFree(va.p);
     va.p = nullptr;
     const uint64_t *sorted_keys = dk.Current();
@@ -1408,7 +1458,7 @@ int set_dets(sci_ctx *ctx, const uint64_t *keys, int nwords, int64_t M, int n_al
             auto kf = nwords == 4 ? k_fill2<4> : nwords == 3 ? k_fill2<3> : nwords == 2 ? k_fill2<2> : k_fill2<1>;
             kf<<<grid_for(B.kept * 32), 256, 0, st>>>(B.order.as<uint32_t>(), B.counts.as<uint32_t>(),
                                                           B.offsets.as<uint32_t>(), B.newoff.as<uint32_t>(),
-                                                          B.ukeys.as<uint64_t>(), B.vals_sorted.as<uint64_t>(), B.kept,
+                                                          B.ukeys.as<uint64_t>(), B.vals_sorted.p, ctx->keys, B.kept,
                                                           ctx->e2_idx, ctx->e2_code, ctx->e2_pos);
             SCI_CK(cudaGetLastError());
         }
@@ -1429,7 +1479,7 @@ int set_dets(sci_ctx *ctx, const uint64_t *keys, int nwords, int64_t M, int n_al
             auto kf = nwords == 4 ? k_fill1<4> : nwords == 3 ? k_fill1<3> : nwords == 2 ? k_fill1<2> : k_fill1<1>;
             kf<<<grid_for(B.kept * 32), 256, 0, st>>>(B.order.as<uint32_t>(), B.counts.as<uint32_t>(),
                                                           B.offsets.as<uint32_t>(), B.newoff.as<uint32_t>(),
-                                                          B.ukeys.as<uint64_t>(), B.vals_sorted.as<uint64_t>(), B.kept,
+                                                          B.ukeys.as<uint64_t>(), B.vals_sorted.p, ctx->keys, B.kept,
                                                           ctx->e1_idx, ctx->e1_S, ctx->e1_meta);
             SCI_CK(cudaGetLastError());
         }
