@@ -781,7 +781,7 @@ int order_runs(sci_ctx *ctx, int nruns, Buckets &B)
 }
 
 // ------------------------------------------------------------------ size bounds
-// The (N-2) table holds its buckets largest first, so the buckets of more than thr members
+// The (N-2) table holds whole buckets, largest first, so the buckets of more than thr members
 // are its first entries.  Thread t finds the end of that prefix for its threshold by
 // bisection: out[t], and the bucket size found there (0 at the end of the table) in out[n + t].
 struct Thresholds {
@@ -799,6 +799,24 @@ __global__ void k_size_bounds(const uint32_t *__restrict__ e_pos, int64_t E, Thr
     }
     out[t] = lo;
     out[q.n + t] = lo < E ? sci::pos_size(e_pos[lo]) : 0;
+}
+
+// *bad = 1 unless the table holds whole buckets of two and more members in order of falling
+// size: the bisection above and the kernels that read runs of equal buckets rely on it.
+__global__ void k_check_order(const uint32_t *__restrict__ e_pos, int64_t E, int64_t *bad)
+{
+    bool ok = true;
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < E; p += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t pos = e_pos[p];
+        const int off = sci::pos_off(pos), size = sci::pos_size(pos);
+        ok &= size >= 2 && (p > 0 || off == 0);
+        if (off + 1 < size) {
+            ok &= p + 1 < E && e_pos[p + 1] == pos + 1;
+        } else {
+            ok &= off + 1 == size && (p + 1 == E || (sci::pos_off(e_pos[p + 1]) == 0 && sci::pos_size(e_pos[p + 1]) <= size));
+        }
+    }
+    if (!ok) *bad = 1;
 }
 
 // tile starts: the entries at bucket offsets 0, kTileRows, 2 kTileRows, ...
@@ -824,28 +842,37 @@ void sci_free_split(sci_ctx *ctx, bool ranged)
     sp = sci::TileSplit{};
 }
 
-int sci_table_split(sci_ctx *ctx, bool ranged)
+namespace {
+// the split of the full or the range table at the context's threshold; on failure the context
+// and `out` are as they were
+int make_split(sci_ctx *ctx, bool ranged, sci::TileSplit &out)
 {
-    sci_free_split(ctx, ranged);
     const uint32_t *e_pos = ranged ? ctx->r2_pos : ctx->e2_pos;
     const int64_t E = ranged ? ctx->r2 : ctx->e2;
-    if (E == 0) return SCI_OK;
-    cudaStream_t st = ctx->stream;
     sci::TileSplit sp;
+    if (E == 0) {
+        out = sp;
+        return SCI_OK;
+    }
+    cudaStream_t st = ctx->stream;
     const int thr_wide = ctx->tile_user ? ctx->tile_b : std::min(ctx->tile_b, sci::kTileBucketWide);
     Thresholds q;
     q.n = sci::kSortBucket + 3;
     q.thr[0] = ctx->tile_b, q.thr[1] = thr_wide;
     for (int k = 0; k <= sci::kSortBucket; k++) q.thr[2 + k] = k;
-    int64_t h[2 * (sci::kSortBucket + 3)];
+    int64_t h[2 * (sci::kSortBucket + 3) + 1];   // the bounds, the sizes there, the order check
     {
-        TmpBuf out;
-        SCI_CK(cudaMalloc(&out.p, sizeof h));
-        k_size_bounds<<<1, 96, 0, st>>>(e_pos, E, q, out.as<int64_t>());
+        TmpBuf out_dev;
+        SCI_CK(cudaMalloc(&out_dev.p, sizeof h));
+        int64_t *bad = out_dev.as<int64_t>() + 2 * q.n;
+        SCI_CK(cudaMemsetAsync(bad, 0, sizeof *bad, st));
+        k_check_order<<<grid_for(E), 256, 0, st>>>(e_pos, E, bad);
+        k_size_bounds<<<1, 96, 0, st>>>(e_pos, E, q, out_dev.as<int64_t>());
         SCI_CK(cudaGetLastError());
-        SCI_CK(cudaMemcpyAsync(h, out.p, sizeof h, cudaMemcpyDeviceToHost, st));
+        SCI_CK(cudaMemcpyAsync(h, out_dev.p, sizeof h, cudaMemcpyDeviceToHost, st));
         SCI_CK(cudaStreamSynchronize(st));
     }
+    if (h[2 * q.n]) return sci_fail(ctx, SCI_ERR_STATE, "internal: (N-2) buckets not in size order");
     sp.base.big = h[0], sp.base.maxb_small = (int)h[q.n];
     sp.wide.big = h[1], sp.wide.maxb_small = (int)h[q.n + 1];
     for (int k = 0; k <= sci::kSortBucket; k++) sp.above[k] = h[2 + k];
@@ -877,6 +904,17 @@ int sci_table_split(sci_ctx *ctx, bool ranged)
             return sci_cuda_check(ctx, e, "tile list");
         }
     }
+    out = sp;
+    return SCI_OK;
+}
+}  // namespace
+
+int sci_table_split(sci_ctx *ctx, bool ranged)
+{
+    sci::TileSplit sp;
+    const int rc = make_split(ctx, ranged, sp);
+    if (rc != SCI_OK) return rc;
+    sci_free_split(ctx, ranged);
     (ranged ? ctx->rsplit2 : ctx->split2) = sp;
     return SCI_OK;
 }
@@ -1360,15 +1398,21 @@ extern "C" int sci_set_tile_threshold(sci_ctx *ctx, int members)
     ctx->tile_b = members == 0 ? sci::kTileBucket : members;
     ctx->tile_user = members != 0;
     if (!ctx->have_dets) return SCI_OK;
-    int rc = sci_table_split(ctx, false);
-    if (rc == SCI_OK && ctx->ranged) rc = sci_table_split(ctx, true);
+    // both new splits before either old one goes: a call that fails changes nothing
+    sci::TileSplit full, range;
+    int rc = make_split(ctx, false, full);
+    if (rc == SCI_OK && ctx->ranged) rc = make_split(ctx, true, range);
+    std::swap(ctx->split2, full);
     if (rc == SCI_OK && !sci_sigma_window_fits(ctx))
         rc = sci_fail(ctx, SCI_ERR_OVERFLOW, "buckets left to the window kernels do not fit shared memory");
-    if (rc != SCI_OK) {   // back to the previous threshold, whose split was valid
+    if (rc != SCI_OK) {   // back to the previous threshold and its split
         ctx->tile_b = old, ctx->tile_user = old_user;
-        sci_table_split(ctx, false);
-        if (ctx->ranged) sci_table_split(ctx, true);
+        std::swap(ctx->split2, full);
+    } else if (ctx->ranged) {
+        std::swap(ctx->rsplit2, range);
     }
+    if (full.tiles) cudaFree(full.tiles);
+    if (range.tiles) cudaFree(range.tiles);
     return rc;
 }
 
