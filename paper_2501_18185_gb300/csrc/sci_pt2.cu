@@ -69,8 +69,11 @@ struct Pt2 {
     uint64_t ref, ref_hi, ref_w2;   // the reference string: orbitals 0..63, 64..127, 128..191
     const double *tab, *fref, *g_so;
     const double *Eref;
-    const double *fix_scale;  // F and G as integers in units of 1 / fix_scale: [norb], [norb][norb]
+    // F and G as integers in units of 1 / fix_scale[0]: [norb], [norb][norb]; when fix_scale[1]
+    // is not 0, the sums need what the units leave of them (rest, the same layout)
+    const double *fix_scale;
     const long long *fix;
+    const double *rest;
     uint32_t gcode[192];      // codes of the beta orbitals (spin-orbital mode) or spinors
     uint8_t obc[192];         // those orbitals sorted by code
     uint8_t cstart[(1 << kMaxBits) + 1];  // first index in obc of each code
@@ -747,15 +750,37 @@ k_pt2_gen_z(const uint64_t *__restrict__ Pkeys, int64_t M, const zdbl *__restric
 
 // sum over the table entries of num^2 / (E0 - H_II).  Each warp packs the occupied slots
 // it scans into a buffer of 32 and evaluates full buffers, so every lane works.  Instruction
-// issue bounds it, so H_II - E_ref (O(level^2) table terms) is summed as 64-bit integers: F and
-// G in units of 1 / fix_scale, chosen by k_pt2_setup so that no sum overflows (exact sums of
-// terms rounded to 2^-62 of their largest total, two integer adds a term), and the inner
-// loops run over a list of the differing orbitals in shared memory, not over bits.
+// issue bounds it, so H_II - E_ref (O(level^2) table terms) is summed as 64-bit integers, two
+// integer adds a term: F and G in units that k_pt2_setup chooses so that no sum overflows, each
+// rounded by half a unit at most.  The inner loops run over a list of the differing orbitals in
+// shared memory, not over bits.  The units are at most 2^-56 |E_ref|, an eighth of the FP64
+// spacing at E_ref; where the integrals spread too far for that (an orbital shifted out of
+// reach), fix_rest() adds in FP64 what the rounding left, and the sum is that of FP64 again (24
+// orbitals, M = 12k, whole call: 6.8 ms, 8.3 with the rest).
 // Against paired-FP32 sums over bits: 30 orbitals, M = 60k, one root, 2.4e8 determinants 20.4 ->
 // 13.2 ms; 24 orbitals, M = 40k, two roots, 1.4e8 determinants 13.5 -> 12.5 (the FP64 divisions,
 // one a root, bind there).
 // GS: G in shared memory (up to 162 orbitals); else read from global memory.
 constexpr int kDiffList = 32;   // orbitals of the list; determinants that differ in more walk bits
+// the part of H_II - E_ref that the units of the integer sums leave, for holes H and particles P
+template <typename K> __device__ __noinline__ double fix_rest(const double *__restrict__ rest, int norb, K H, K Pm)
+{
+    const double *G = rest + norb;
+    double e = 0.0;
+    for (K m = H; m; m &= m - 1) {
+        const int i = lowbit(m);
+        e -= __ldg(rest + i);
+        for (K m2 = m & (m - 1); m2; m2 &= m2 - 1) e += __ldg(G + i * norb + lowbit(m2));
+        for (K m2 = Pm; m2; m2 &= m2 - 1) e -= __ldg(G + i * norb + lowbit(m2));
+    }
+    for (K m = Pm; m; m &= m - 1) {
+        const int a = lowbit(m);
+        e += __ldg(rest + a);
+        for (K m2 = m & (m - 1); m2; m2 &= m2 - 1) e += __ldg(G + a * norb + lowbit(m2));
+    }
+    return e;
+}
+
 template <int R, bool CPLX, int KW, bool GS = true>
 __global__ void __launch_bounds__(kThreads)
 k_pt2_eval(Pt2 p, uint64_t cap, const double *__restrict__ E0, double *__restrict__ out)
@@ -775,7 +800,8 @@ k_pt2_eval(Pt2 p, uint64_t cap, const double *__restrict__ E0, double *__restric
         if constexpr (GS) return sGs[t];
         else return __ldg(p.fix + norb + t);
     };
-    const double unit = 1.0 / *p.fix_scale;
+    const double unit = 1.0 / p.fix_scale[0];
+    const bool wide = p.fix_scale[1] != 0.0;
     const double Eref = *p.Eref;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     double acc[R], e0[R];
@@ -822,7 +848,9 @@ k_pt2_eval(Pt2 p, uint64_t cap, const double *__restrict__ E0, double *__restric
                 for (K m2 = m & (m - 1); m2; m2 &= m2 - 1) e += gget(a * norb + lowbit(m2));
             }
         }
-        const double hii = Eref + (double)e * unit;
+        double de = (double)e * unit;
+        if (wide) de += fix_rest<K>(p.rest, norb, H, Pm);
+        const double hii = Eref + de;
 #pragma unroll
         for (int v = 0; v < R; v++) {
             double num2;
@@ -915,11 +943,12 @@ k_pt2_p(int64_t M, const T *__restrict__ C, const T *__restrict__ S, const doubl
 __device__ __forceinline__ double re_of(double a) { return a; }
 __device__ __forceinline__ double re_of(zdbl a) { return a.x; }
 
+// dmax: the most orbitals in which a determinant differs from the reference
 template <typename T>
-__global__ void k_pt2_setup(int norb, uint64_t ref_lo, uint64_t ref_hi, uint64_t ref_w2, const T *__restrict__ h_so,
+__global__ void k_pt2_setup(int norb, int dmax, uint64_t ref_lo, uint64_t ref_hi, uint64_t ref_w2, const T *__restrict__ h_so,
                             const T *__restrict__ jd, const T *__restrict__ kd, double *__restrict__ G,
                             double *__restrict__ fdiag, double *__restrict__ Eref, double *__restrict__ fix_scale,
-                            long long *__restrict__ fix)
+                            long long *__restrict__ fix, double *__restrict__ rest)
 {
     __shared__ unsigned long long s_max[2];   // largest |F| and |G|, as bits (ordered like the values)
     if (threadIdx.x < 2) s_max[threadIdx.x] = 0ull;
@@ -938,15 +967,21 @@ __global__ void k_pt2_setup(int norb, uint64_t ref_lo, uint64_t ref_hi, uint64_t
         atomicMax(&s_max[0], (unsigned long long)__double_as_longlong(fabs(f)));
     }
     __syncthreads();
-    // F and G as integers: the largest power of two that keeps any sum of them below 2^62
-    const double bound = norb * __longlong_as_double((long long)s_max[0]) +
-                         0.5 * norb * norb * __longlong_as_double((long long)s_max[1]);
+    // F and G as integers: the largest power of two that keeps any sum of them below 2^62 (the
+    // terms of dmax orbitals and of their pairs).  Integrals whose sums overflow FP64 give NaN.
+    const double d = max(dmax, 2);
+    const double bound = d * __longlong_as_double((long long)s_max[0]) +
+                         0.5 * d * (d - 1.0) * __longlong_as_double((long long)s_max[1]);
     int ex = 0;
     frexp(bound, &ex);   // bound < 2^ex
-    const double scale = ldexp(1.0, min(62 - ex, 1000));
-    if (threadIdx.x == 0) *fix_scale = scale;
-    for (int t = threadIdx.x; t < norb; t += blockDim.x) fix[t] = llrint(fdiag[t] * scale);
-    for (int t = threadIdx.x; t < norb * norb; t += blockDim.x) fix[norb + t] = llrint(G[t] * scale);
+    const double scale = bound <= 1.7976931348623157e308 ? ldexp(1.0, min(62 - ex, 1000)) : nan(""), unit = 1.0 / scale;
+    auto split = [&](double x, int at) {
+        const double u = x * scale;
+        fix[at] = llrint(u);
+        rest[at] = (u - (double)fix[at]) * unit;   // exact: u has 53 bits, and none left from 2^53 on
+    };
+    for (int t = threadIdx.x; t < norb; t += blockDim.x) split(fdiag[t], t);
+    for (int t = threadIdx.x; t < norb * norb; t += blockDim.x) split(G[t], norb + t);
     if (threadIdx.x == 0) {
         double e = 0.0;
         for (W3 m = ref; m; m &= m - 1) {
@@ -955,6 +990,8 @@ __global__ void k_pt2_setup(int norb, uint64_t ref_lo, uint64_t ref_hi, uint64_t
             for (W3 m2 = m & (m - 1); m2; m2 &= m2 - 1) e += G[i * norb + lowbit(m2)];
         }
         *Eref = e;
+        fix_scale[0] = scale;
+        fix_scale[1] = unit > ldexp(fabs(e), -56) ? 1.0 : 0.0;
     }
 }
 
@@ -1025,7 +1062,7 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
         if (tab2) cudaFree(tab2);
         if (bnd_free) cudaFree(bnd_free);
     };
-    const size_t nsmall = (size_t)R * 3 + 2 * ((size_t)norb * norb + norb) + 2 + 2;
+    const size_t nsmall = (size_t)R * 3 + 3 * ((size_t)norb * norb + norb) + 3 + 2;
     if (cudaMalloc(&S, sizeof(double) * SC * std::max<int64_t>(1, M) * R) != cudaSuccess ||
         cudaMalloc(&small, sizeof(double) * nsmall) != cudaSuccess) {
         cleanup();
@@ -1034,7 +1071,8 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
     double *dE0 = small, *outW = small + R, *outP = small + 2 * R, *G = small + 3 * R, *fdiag = G + norb * norb,
            *Eref = fdiag + norb;
     double *fix_scale = Eref + 1;
-    long long *fix = reinterpret_cast<long long *>(fix_scale + 1);
+    double *rest = fix_scale + 2;
+    long long *fix = reinterpret_cast<long long *>(rest + norb * norb + norb);
     unsigned long long *count = reinterpret_cast<unsigned long long *>(fix + norb * norb + norb);
     int *flag = reinterpret_cast<int *>(count + 1);
     if (sci_cuda_check(ctx, cudaMemsetAsync(small, 0, sizeof(double) * nsmall, st), "enpt2 memset") ||
@@ -1055,12 +1093,13 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
         else
             k_pt2_p<R, double><<<grid_for(M), kThreads, 0, st>>>(M, C, S, ctx->hdiag, dE0, outP);
     }
+    const int dmax = 2 * (ctx->spinors ? std::min(ctx->N, n - ctx->N) : std::min(na, n - na) + std::min(nb, n - nb));
     if constexpr (SPIN)
-        k_pt2_setup<zdbl><<<1, 256, 0, st>>>(norb, ctx->ref, ctx->ref_hi, ctx->ref_w2, (const zdbl *)ctx->h_so,
-                                             (const zdbl *)ctx->jd, (const zdbl *)ctx->kd, G, fdiag, Eref, fix_scale, fix);
+        k_pt2_setup<zdbl><<<1, 256, 0, st>>>(norb, dmax, ctx->ref, ctx->ref_hi, ctx->ref_w2, (const zdbl *)ctx->h_so,
+                                             (const zdbl *)ctx->jd, (const zdbl *)ctx->kd, G, fdiag, Eref, fix_scale, fix, rest);
     else
-        k_pt2_setup<double><<<1, 256, 0, st>>>(norb, ctx->ref, ctx->ref_hi, ctx->ref_w2, (const double *)ctx->h_so,
-                                               (const double *)ctx->jd, (const double *)ctx->kd, G, fdiag, Eref, fix_scale, fix);
+        k_pt2_setup<double><<<1, 256, 0, st>>>(norb, dmax, ctx->ref, ctx->ref_hi, ctx->ref_w2, (const double *)ctx->h_so,
+                                               (const double *)ctx->jd, (const double *)ctx->kd, G, fdiag, Eref, fix_scale, fix, rest);
     // the table: capacity a power of two within the budget
     const size_t slot = sizeof(uint64_t) * SW;
     uint64_t cap = 1ull << 8;  // at least 256 entries
@@ -1109,7 +1148,7 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
     }
     p.n = n, p.norb = norb, p.na = na, p.nb = nb, p.ref = ctx->ref, p.ref_hi = ctx->ref_hi, p.ref_w2 = ctx->ref_w2;
     p.tab = (const double *)ctx->tab, p.fref = (const double *)ctx->fref, p.g_so = (const double *)ctx->g_so;
-    p.Eref = Eref, p.fix_scale = fix_scale, p.fix = fix;
+    p.Eref = Eref, p.fix_scale = fix_scale, p.fix = fix, p.rest = rest;
     p.tab2 = tab2, p.mask = cap - 1, p.count = count, p.flag = flag;
     p.limit = (unsigned long long)(0.85 * (double)cap);
     p.eps = eps;
