@@ -16,15 +16,16 @@
 //     Wt = sum w_I, D = sum w_I Delta(I), DD = sum w_I Delta Delta^T,
 //     accumulated per CTA in shared memory.
 //   singles (members X = S + x, Y = S + y of one (N-1) bucket): w = conj(c_X) c_Y ph,
-//     g1[x][y] += w, and for every spectator k in S
+//     g1[x][y] += w, and for every spectator k in S (A and Bc below take every unordered
+//     pair in one orientation, and the expansion adds the conjugate)
 //       g2[x][y][k][k] = g2[k][k][x][y] = -g2[x][k][k][y] = -g2[k][y][x][k] += w.
 //     The spectator sum b[x][y][k] = sum w n_k(S) is kept as A[x][y] n_k(ref) + Bc[x][y][k]
 //     with Bc taking only the orbitals of S that differ from the reference (the same
 //     reference decomposition as the sigma singles).
 //   doubles (members I = K + {a,b}, J = K + {i,j} of one (N-2) bucket, disjoint): one
 //     atomic add of w = conj(c_I) c_J ph into a table laid out like the pair-integral
-//     table (with separate alpha-alpha and beta-beta regions), for the pairs with the
-//     bra before the ket in the bucket; the other orientation is its conjugate.  Then
+//     table (with separate alpha-alpha and beta-beta regions), every unordered pair in one
+//     of its two orientations; the other is its conjugate.  Then
 //       g2[a][i][b][j] = g2[b][j][a][i] = -g2[a][j][b][i] = -g2[b][i][a][j]
 //         = dT[bra, ket] + conj(dT[ket, bra]).
 // Signs: <I| a+_a a+_b a_j a_i |J> is the phase (-1)^(pi_I + pi_J) of the sigma kernels.
@@ -530,28 +531,60 @@ template <typename TC> struct Tables {
     }
 };
 
-template <typename TC> __global__ void k_rdm_expand1(Tables<TC> T, TC *__restrict__ g1)
+// g1 and, after k_rdm_expand2, the elements of g2 of the other two classes, n^3 of its n^4: a
+// thread per (x, y, k), per (x, y) when g2 is null.
+template <typename TC> __global__ void k_rdm_expand1(Tables<TC> T, TC *__restrict__ g1, TC *__restrict__ g2)
 {
-    const int n2 = T.norb * T.norb;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n2; t += gridDim.x * blockDim.x) {
-        const int x = t / T.norb, y = t % T.norb;
-        g1[t] = x == y ? from_real<TC>(T.pair_occ(x, x)) : T.single(x, y);
+    const int norb = T.norb, kk = g2 ? norb : 1;
+    const int64_t n2 = (int64_t)norb * norb, n3 = n2 * norb;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n2 * kk; t += (int64_t)gridDim.x * blockDim.x) {
+        const int k = (int)(t % kk), xy = (int)(t / kk), x = xy / norb, y = xy % norb;
+        if (k == 0) g1[xy] = x == y ? from_real<TC>(T.pair_occ(x, x)) : T.single(x, y);
+        if (!g2 || x == y) continue;
+        if (k == x) {
+            const double o = T.pair_occ(x, y);
+            g2[x * n3 + x * n2 + y * norb + y] = from_real<TC>(o);      // (x x | y y)
+            g2[x * n3 + y * n2 + y * norb + x] = from_real<TC>(-o);     // (x y | y x)
+        } else if (k != y && T.spin(x) == T.spin(y)) {
+            const TC b = T.spectator(x, y, k);
+            g2[x * n3 + y * n2 + k * norb + k] = b;          // (x y | k k)
+            g2[k * n3 + k * n2 + x * norb + y] = b;          // (k k | x y)
+            g2[x * n3 + k * n2 + k * norb + y] = neg(b);     // (x k | k y)
+            g2[k * n3 + y * n2 + x * norb + k] = neg(b);     // (k y | x k)
+        }
     }
 }
 
-// g2, every element once in storage order: a CTA takes the [r][s] matrices of its (p, q), so
-// that the writes, which bound it (norb^4 elements, 104 MB at 60 spin-orbitals), are
-// consecutive and g2 needs no clearing; the tables are small and read from L2.
-// 118 us at 60 spin-orbitals, where the clear and the scattered stores of one thread per table
-// entry took 100; the gradients, which sum straight from the tables, no longer form g2.  (Adding
-// the two orientations in a pass of its own first: 122 us for both.)
+// The double excitations of g2, and zeros elsewhere: every element once in storage order, so that
+// g2 needs no clearing.  A CTA takes a (p, q), a warp one row r at a time and its lanes s: what
+// belongs to the bra and the spin of s are the warp's, and a row that conserves no spin is only
+// stored.  The elements of the other classes are left to k_rdm_expand1: one of them in a warp's
+// 32 cost its five to eight FP64 instructions, 16 cycles of the pipe each, as if all were.
+// Both kernels at 60 spin-orbitals: 47 us, 118 in one kernel with all classes (a clear and
+// scattered stores of all classes took 100); the writes alone, 104 MB, 15 us.
 template <typename TC> __global__ void __launch_bounds__(kThreads) k_rdm_expand2(Tables<TC> T, TC *__restrict__ g2)
 {
     const int norb = T.norb, n2 = norb * norb;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int pq = blockIdx.x; pq < n2; pq += gridDim.x) {
-        const int p = pq / norb, q = pq % norb;
-        TC *out = g2 + (int64_t)pq * n2;
-        for (int t = threadIdx.x; t < n2; t += blockDim.x) out[t] = T.two(p, q, t / norb, t % norb);
+        const int p = pq / norb, q = pq % norb, ds = T.spin(p) - T.spin(q);
+        for (int r = wid; r < norb; r += kThreads / 32) {
+            TC *out = g2 + ((int64_t)pq * norb + r) * norb;
+            const int ss = ds + T.spin(r);   // the spin of s, by conservation
+            const bool any = p != q && p != r && r != q;
+            uint32_t row = 0, col2 = 0;
+            if (any) grad_offsets(T.tr, min(p, r), max(p, r), T.bb_off, row, col2);
+            for (int s = lane; s < norb; s += 32) {
+                TC v = from_real<TC>(0.0);
+                if (any && s != p && s != q && s != r && T.spin(s) == ss) {
+                    uint32_t row2, col;
+                    grad_offsets(T.tr, min(q, s), max(q, s), T.bb_off, row2, col);
+                    v = add(T.dT[(int64_t)row + col], conjv(T.dT[(int64_t)row2 + col2]));
+                    if ((p < r) != (q < s)) v = neg(v);
+                }
+                out[s] = v;
+            }
+        }
     }
 }
 
@@ -702,8 +735,8 @@ int rdm_run(sci_ctx *ctx, const TC *C, int nvec, const double *wk_dev, TC *g1, T
     const int rc = rdm_tables<TC>(ctx, C, nvec, wk_dev, g2 != nullptr, T);
     if (rc) return rc;
     const int n2 = ctx->norb * ctx->norb;
-    k_rdm_expand1<TC><<<grid_for(n2), kThreads, 0, ctx->stream>>>(T, g1);
     if (g2) k_rdm_expand2<TC><<<n2, kThreads, 0, ctx->stream>>>(T, g2);
+    k_rdm_expand1<TC><<<grid_for((int64_t)n2 * (g2 ? ctx->norb : 1)), kThreads, 0, ctx->stream>>>(T, g1, g2);
     return sci_cuda_check(ctx, cudaGetLastError(), "rdm12 launch") ? SCI_ERR_CUDA : SCI_OK;
 }
 
