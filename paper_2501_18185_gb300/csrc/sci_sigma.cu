@@ -420,6 +420,13 @@ template <class P, int NV> constexpr int sort_from(bool small_table)
     if (!P::kFp64) return kSortBucket + 1;
     return NV == 1 && sizeof(typename P::SC) == sizeof(double) && !small_table ? 33 : kSmallBucket + 1;
 }
+// Entries of the buckets of at most kSortBucket members up to which the paired-FP32 and
+// FP32-storage launches take them in the aligned walk of the larger ones instead of by size: a
+// launch costs about 2 us, and these policies gain less by size than FP64 does.  Two
+// paired-FP32 vectors, the product: 30 orbitals, 1,000 determinants (76k entries) 70 us by size,
+// 43 in one walk; 3,000 (118k) 75, 45; full CI of 8 orbitals (137k) 51, 45; 40 orbitals, M =
+// 60k, one vector (922k) 209, 228; FP32 storage at 8 vectors, 221k entries 51, 60.
+constexpr int64_t kFewEntries = 200'000;
 // The tiled walk takes 32 columns at a time as a mask of doubles for complex FP64 (64
 // spinors, M = 500k: 1.43 -> 1.25 ms) and one FP64 vector (70 orbitals, M = 120k: doubles
 // 1.25 -> 1.02 ms); otherwise in aligned groups (40 orbitals, two vectors: 1.22 ms, 1.29 by
@@ -1234,8 +1241,8 @@ int launch_tiled(sci_ctx *ctx, const Tabs &T, const sci::Split &sp, const typena
 template <bool RG> constexpr size_t row_extra() { return RG ? 8 + sizeof(uint16_t) : 8; }
 
 // the doubles of one vector group, by bucket size: the tiled kernel above the tile threshold,
-// the aligned walk down to kSortBucket members, then the sorted kernel, the aligned walk
-// and the register kernel as sort_from() and kSmallBucket say
+// the aligned walk down to kSortBucket members (or to the end, see kFewEntries), then the sorted
+// kernel, the aligned walk and the register kernel as sort_from() and kSmallBucket say
 template <class P, bool RG, bool ST, int NV>
 int launch_doubles(sci_ctx *ctx, const Tabs &T, const typename P::TT *tab, const typename P::CI *C, int nvec, int v0,
                    typename P::TO *S, bool &chained)
@@ -1264,7 +1271,8 @@ int launch_doubles(sci_ctx *ctx, const Tabs &T, const typename P::TT *tab, const
     // the first entry of each part: the tiles end at b, the middle buckets at m, the sorted
     // ones at so, the aligned ones of five members and more at sm
     const int64_t *above = T.ts->above;
-    const int64_t b = sp.big, m = std::max(b, above[kSortBucket]);
+    const int64_t b = sp.big, large = std::max(b, above[kSortBucket]);
+    const int64_t m = !P::kFp64 && T.e2 - large <= kFewEntries ? T.e2 : large;
     constexpr int lowest = sort_from<P, NV>(true);
     const int from = sort_from<P, NV>(ctx->tab_elems * (int64_t)sizeof(typename P::TT) <= kSmallTable);
     const int64_t sm = lowest <= kSmallBucket ? T.e2 : std::max(m, above[kSmallBucket]);
