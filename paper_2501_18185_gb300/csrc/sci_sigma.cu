@@ -427,6 +427,18 @@ template <class P, int NV> constexpr int sort_from(bool small_table)
 // 43 in one walk; 3,000 (118k) 75, 45; full CI of 8 orbitals (137k) 51, 45; 40 orbitals, M =
 // 60k, one vector (922k) 209, 228; FP32 storage at 8 vectors, 221k entries 51, 60.
 constexpr int64_t kFewEntries = 200'000;
+// ... and in a row range in FP32 storage, when the space has larger buckets too: a short range
+// owns few of a bucket's rows, and the launches by size stage and sort the others all the same.
+// M = 400k, a 64th of the rows, 8 vectors (1.4M entries): 153 us by size, 140; M = 60k, an eighth,
+// one vector (2.5M): 91, 84; M = 400k, an eighth, one vector (6.5M): 143, 162.  (Without larger
+// buckets the windows are too short for the rows they own: full CI of 10 orbitals, a 64th, 8
+// vectors, 221k entries: 51, 60.)
+constexpr int64_t kFewRangeEntries = 3'000'000;
+template <class P, bool RANGED> constexpr int64_t few_entries(bool larger)
+{
+    if (P::kFp64) return 0;
+    return RANGED && !P::kSplit && larger ? kFewRangeEntries : kFewEntries;
+}
 // The tiled walk takes 32 columns at a time as a mask of doubles for complex FP64 (64
 // spinors, M = 500k: 1.43 -> 1.25 ms) and one FP64 vector (70 orbitals, M = 120k: doubles
 // 1.25 -> 1.02 ms); otherwise in aligned groups (40 orbitals, two vectors: 1.22 ms, 1.29 by
@@ -1272,7 +1284,7 @@ int launch_doubles(sci_ctx *ctx, const Tabs &T, const typename P::TT *tab, const
     // ones at so, the aligned ones of five members and more at sm
     const int64_t *above = T.ts->above;
     const int64_t b = sp.big, large = std::max(b, above[kSortBucket]);
-    const int64_t m = !P::kFp64 && T.e2 - large <= kFewEntries ? T.e2 : large;
+    const int64_t m = T.e2 - large <= few_entries<P, RG>(large > b) ? T.e2 : large;
     constexpr int lowest = sort_from<P, NV>(true);
     const int from = sort_from<P, NV>(ctx->tab_elems * (int64_t)sizeof(typename P::TT) <= kSmallTable);
     const int64_t sm = lowest <= kSmallBucket ? T.e2 : std::max(m, above[kSmallBucket]);

@@ -90,3 +90,21 @@ def test_dispatch(gpu, name):
             H.set_deterministic(0)
             assert np.array_equal(D1, D2)
             assert np.abs(D1 - S).max() <= 1e-13 * np.abs(S).max()
+
+
+def test_short_ranges(gpu):
+    """Row ranges of a few rows, whose tables in FP32 storage take one walk where the whole list
+    goes by size, and of most rows."""
+    torch = gpu
+    w = SPACES["all_sizes"]()
+    H = sci.Hamiltonian.from_workload(w)
+    for nvec in (1, 3, 8):
+        t = torch.from_numpy(np.ascontiguousarray(w.c[:, :nvec])).cuda().float()
+        S = H.sigma(t, prec=sci.SCI_PREC_F32_STORE_F64_ACC)
+        for a, b in ((0, 1), (w.M // 2, w.M // 2 + 64), (w.M - 5000, w.M), (1, w.M)):
+            part = torch.full((w.M, nvec), 7.0, dtype=torch.float64, device="cuda")
+            H.set_row_range(a, b)
+            H.sigma(t, out=part, prec=sci.SCI_PREC_F32_STORE_F64_ACC)
+            H.set_row_range(0, w.M)
+            assert (part[a:b] - S[a:b]).abs().max() <= 1e-13 * S.abs().max()
+            assert (part[:a] == 7.0).all() and (part[b:] == 7.0).all()
