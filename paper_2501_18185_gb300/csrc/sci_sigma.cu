@@ -404,7 +404,8 @@ inline int window_rows(int64_t entries, int rows)
 // The smallest bucket of the sorted kernel.  It pays where the products bind: FP64 at two and
 // more vectors or complex (64 spinors, M = 500k, 5 to 64 members: 2.15 ms aligned, 1.41 ms
 // sorted; 40 orbitals, two vectors: 0.83, 0.74; 30 orbitals at M = 500k, four vectors, whole
-// kernel: 2.84, 2.60).  One FP64 vector is bound by the table gathers too, and the sort
+// kernel: 2.84, 2.60; whole products of 8 vectors, aligned up to 32 members against sorted: M =
+// 400k 4.76, 4.58; M = 60k 1.87, 1.86; 14 orbitals 0.76, 0.69).  One FP64 vector is bound by the table gathers too, and the sort
 // scatters a bucket's rows over warps: 33 to 64 members gain on the 60k space (206 -> 165 us)
 // and lose little on the 2M one (2.78 -> 2.85 ms), smaller ones lose (2M: 3.48 ms from 5 on).
 // The paired-FP32 sums (27 orbitals, one vector: 216 us aligned, 279 sorted; FP32 storage at
@@ -412,8 +413,10 @@ inline int window_rows(int64_t entries, int rows)
 // instruction issue, sorts all buckets (30 orbitals, M = 500k: 2.48 ms aligned, 2.37 sorted,
 // 2.44 with the register kernel's eight lanes per small bucket).
 // A pair table of kSmallTable bytes or less stays close to the SMs, and one FP64 vector then
-// sorts from 5 members on too (full CI of 10 orbitals: 162 -> 131 us).
-constexpr int64_t kSmallTable = 1 << 20;
+// sorts from 5 members on too (full CI of 10 orbitals, 0.1 MB: 245 us aligned, 228 sorted; 12
+// orbitals, M = 20k, 0.24 MB: 63, 56).  Above it the aligned walk is the faster one again (M = 60k:
+// 14 orbitals, 0.37 MB 142, 145; 16, 0.64 MB 110, 121; 18, 0.97 MB 101, 108).
+constexpr int64_t kSmallTable = 1 << 18;
 template <class P, int NV> constexpr int sort_from(bool small_table)
 {
     if (f32_wide<P, NV>()) return 2;
