@@ -69,11 +69,11 @@ struct Pt2 {
     uint64_t ref, ref_hi, ref_w2;   // the reference string: orbitals 0..63, 64..127, 128..191
     const double *tab, *fref, *g_so;
     const double *Eref;
-    // F and G as integers in units of 1 / fix_scale[0]: [norb], [norb][norb]; when fix_scale[1]
-    // is not 0, the sums need what the units leave of them (rest, the same layout)
+    const double *fdiag, *G;  // F and G: [norb], [norb][norb]
+    // F and G as integers in units of 1 / fix_scale[0], the same layout, [norb] then [norb][norb];
+    // fix_scale[1] is not 0 when those units are too coarse
     const double *fix_scale;
     const long long *fix;
-    const double *rest;
     uint32_t gcode[192];      // codes of the beta orbitals (spin-orbital mode) or spinors
     uint8_t obc[192];         // those orbitals sorted by code
     uint8_t cstart[(1 << kMaxBits) + 1];  // first index in obc of each code
@@ -748,38 +748,54 @@ k_pt2_gen_z(const uint64_t *__restrict__ Pkeys, int64_t M, const zdbl *__restric
     add_claims(p, nclaim, lane);
 }
 
-// sum over the table entries of num^2 / (E0 - H_II).  Each warp packs the occupied slots
-// it scans into a buffer of 32 and evaluates full buffers, so every lane works.  Instruction
+// evaluate(s) for every occupied slot s of the table, by whole warps: a warp packs the occupied
+// slots that it scans into its buffer `buf` of 64, and evaluates 32 at a time
+template <int KW, typename F>
+__device__ __forceinline__ void each_occupied(const Pt2 &p, uint64_t cap, int SW, uint64_t *buf, F evaluate)
+{
+    const int lane = threadIdx.x & 31;
+    int nbuf = 0;  // occupied slots waiting in the buffer (warp-uniform)
+    const uint64_t stride = (uint64_t)gridDim.x * kThreads;
+    for (uint64_t s0 = (uint64_t)blockIdx.x * kThreads + (uint64_t)(threadIdx.x & ~31); s0 < cap; s0 += stride) {
+        const uint64_t s = s0 + lane;
+        bool occ = false;
+        if (s < cap) {
+            const uint64_t *slot = p.tab2 + s * SW;
+            occ = KW == 1 ? slot[0] != kEmpty : KW == 2 ? (slot[0] | slot[1]) != kEmpty : slot[2] != 0;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, occ);
+        if (occ) buf[nbuf + __popc(m & ((1u << lane) - 1))] = s;
+        nbuf += __popc(m);
+        __syncwarp();
+        if (nbuf >= 32) {
+            evaluate(buf[lane]);
+            __syncwarp();
+            if (lane < nbuf - 32) buf[lane] = buf[32 + lane];
+            nbuf -= 32;
+            __syncwarp();
+        }
+    }
+    if (lane < nbuf) evaluate(buf[lane]);
+}
+template <int KW> __device__ __forceinline__ typename KeyOf<KW>::T slot_key(const uint64_t *slot)
+{
+    if constexpr (KW == 1) return slot[0];
+    else if constexpr (KW == 2) return W2(slot[0], slot[1]);
+    else return W3(slot[0], slot[1], ~slot[2]);
+}
+
+// sum over the table entries of num^2 / (E0 - H_II).  Instruction
 // issue bounds it, so H_II - E_ref (O(level^2) table terms) is summed as 64-bit integers, two
 // integer adds a term: F and G in units that k_pt2_setup chooses so that no sum overflows, each
 // rounded by half a unit at most.  The inner loops run over a list of the differing orbitals in
 // shared memory, not over bits.  The units are at most 2^-56 |E_ref|, an eighth of the FP64
 // spacing at E_ref; where the integrals spread too far for that (an orbital shifted out of
-// reach), fix_rest() adds in FP64 what the rounding left, and the sum is that of FP64 again (24
-// orbitals, M = 12k, whole call: 6.8 ms, 8.3 with the rest).
+// reach), this kernel sets flag[1] and leaves the table to k_pt2_eval64.
 // Against paired-FP32 sums over bits: 30 orbitals, M = 60k, one root, 2.4e8 determinants 20.4 ->
 // 13.2 ms; 24 orbitals, M = 40k, two roots, 1.4e8 determinants 13.5 -> 12.5 (the FP64 divisions,
 // one a root, bind there).
 // GS: G in shared memory (up to 162 orbitals); else read from global memory.
 constexpr int kDiffList = 32;   // orbitals of the list; determinants that differ in more walk bits
-// the part of H_II - E_ref that the units of the integer sums leave, for holes H and particles P
-template <typename K> __device__ __noinline__ double fix_rest(const double *__restrict__ rest, int norb, K H, K Pm)
-{
-    const double *G = rest + norb;
-    double e = 0.0;
-    for (K m = H; m; m &= m - 1) {
-        const int i = lowbit(m);
-        e -= __ldg(rest + i);
-        for (K m2 = m & (m - 1); m2; m2 &= m2 - 1) e += __ldg(G + i * norb + lowbit(m2));
-        for (K m2 = Pm; m2; m2 &= m2 - 1) e -= __ldg(G + i * norb + lowbit(m2));
-    }
-    for (K m = Pm; m; m &= m - 1) {
-        const int a = lowbit(m);
-        e += __ldg(rest + a);
-        for (K m2 = m & (m - 1); m2; m2 &= m2 - 1) e += __ldg(G + a * norb + lowbit(m2));
-    }
-    return e;
-}
 
 template <int R, bool CPLX, int KW, bool GS = true>
 __global__ void __launch_bounds__(kThreads)
@@ -792,6 +808,10 @@ k_pt2_eval(Pt2 p, uint64_t cap, const double *__restrict__ E0, double *__restric
     __shared__ uint64_t sbuf[kWarps][64];
     __shared__ double red[kWarps][R];
     __shared__ uint8_t s_diff[kDiffList][kThreads];
+    if (p.fix_scale[1] != 0.0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) p.flag[1] = 1;
+        return;
+    }
     const int norb = p.norb;
     const long long *sF = s_gf, *sGs = s_gf + norb;
     for (int t = threadIdx.x; t < norb * (GS ? norb + 1 : 1); t += blockDim.x) s_gf[t] = p.fix[t];
@@ -801,7 +821,6 @@ k_pt2_eval(Pt2 p, uint64_t cap, const double *__restrict__ E0, double *__restric
         else return __ldg(p.fix + norb + t);
     };
     const double unit = 1.0 / p.fix_scale[0];
-    const bool wide = p.fix_scale[1] != 0.0;
     const double Eref = *p.Eref;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     double acc[R], e0[R];
@@ -810,10 +829,7 @@ k_pt2_eval(Pt2 p, uint64_t cap, const double *__restrict__ E0, double *__restric
     const K ref = ref_of<K>(p);
     auto evaluate = [&](uint64_t s) {
         const uint64_t *slot = p.tab2 + s * SW;
-        K I;
-        if constexpr (KW == 1) I = slot[0];
-        else if constexpr (KW == 2) I = W2(slot[0], slot[1]);
-        else I = W3(slot[0], slot[1], ~slot[2]);
+        const K I = slot_key<KW>(slot);
         const K H = ref & ~I, Pm = I & ~ref;
         long long e = 0;
         if (popck(H) + popck(Pm) <= kDiffList) {
@@ -848,9 +864,7 @@ k_pt2_eval(Pt2 p, uint64_t cap, const double *__restrict__ E0, double *__restric
                 for (K m2 = m & (m - 1); m2; m2 &= m2 - 1) e += gget(a * norb + lowbit(m2));
             }
         }
-        double de = (double)e * unit;
-        if (wide) de += fix_rest<K>(p.rest, norb, H, Pm);
-        const double hii = Eref + de;
+        const double hii = Eref + (double)e * unit;
 #pragma unroll
         for (int v = 0; v < R; v++) {
             double num2;
@@ -865,28 +879,7 @@ k_pt2_eval(Pt2 p, uint64_t cap, const double *__restrict__ E0, double *__restric
             acc[v] += num2 / (e0[v] - hii);
         }
     };
-    int nbuf = 0;  // occupied slots waiting in this warp's buffer (warp-uniform)
-    const uint64_t stride = (uint64_t)gridDim.x * kThreads;
-    for (uint64_t s0 = (uint64_t)blockIdx.x * kThreads + (uint64_t)w * 32; s0 < cap; s0 += stride) {
-        const uint64_t s = s0 + lane;
-        bool occ = false;
-        if (s < cap) {
-            const uint64_t *slot = p.tab2 + s * SW;
-            occ = KW == 1 ? slot[0] != kEmpty : KW == 2 ? (slot[0] | slot[1]) != kEmpty : slot[2] != 0;
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, occ);
-        if (occ) sbuf[w][nbuf + __popc(m & ((1u << lane) - 1))] = s;
-        nbuf += __popc(m);
-        __syncwarp();
-        if (nbuf >= 32) {
-            evaluate(sbuf[w][lane]);
-            __syncwarp();
-            if (lane < nbuf - 32) sbuf[w][lane] = sbuf[w][32 + lane];
-            nbuf -= 32;
-            __syncwarp();
-        }
-    }
-    if (lane < nbuf) evaluate(sbuf[w][lane]);
+    each_occupied<KW>(p, cap, SW, sbuf[w], evaluate);
 #pragma unroll
     for (int v = 0; v < R; v++) {
         double x = acc[v];
@@ -898,6 +891,64 @@ k_pt2_eval(Pt2 p, uint64_t cap, const double *__restrict__ E0, double *__restric
         double x = 0.0;
         for (int i = 0; i < kWarps; i++) x += red[i][threadIdx.x];
         atomicAdd(out + threadIdx.x, x);
+    }
+}
+
+// The same with H_II summed in FP64, for integrals whose spread is too wide for the integer
+// sums: R roots of a table with SW words per slot.  24 orbitals, M = 12k, the whole call: one root
+// 6.9 ms with the integer sums, 7.8 with this kernel; four roots 7.6, 9.2.
+template <bool CPLX, int KW>
+__global__ void __launch_bounds__(kThreads)
+k_pt2_eval64(Pt2 p, uint64_t cap, int R, int SW, const double *__restrict__ E0, double *__restrict__ out)
+{
+    using K = typename KeyOf<KW>::T;
+    __shared__ uint64_t sbuf[kWarps][64];
+    const int norb = p.norb;
+    const double scale = p.fix_scale[0];   // NaN where sums overflow FP64: they give no number
+    const double Eref = scale == scale ? *p.Eref : scale;
+    const K ref = ref_of<K>(p);
+    double acc[8];
+#pragma unroll
+    for (int v = 0; v < 8; v++) acc[v] = 0.0;
+    each_occupied<KW>(p, cap, SW, sbuf[threadIdx.x >> 5], [&](uint64_t s) {
+        const uint64_t *slot = p.tab2 + s * SW;
+        const K I = slot_key<KW>(slot);
+        const K H = ref & ~I, Pm = I & ~ref;
+        double e = 0.0;
+        for (K m = H; m; m &= m - 1) {
+            const int i = lowbit(m);
+            e -= __ldg(p.fdiag + i);
+            for (K m2 = m & (m - 1); m2; m2 &= m2 - 1) e += __ldg(p.G + i * norb + lowbit(m2));
+            for (K m2 = Pm; m2; m2 &= m2 - 1) e -= __ldg(p.G + i * norb + lowbit(m2));
+        }
+        for (K m = Pm; m; m &= m - 1) {
+            const int a = lowbit(m);
+            e += __ldg(p.fdiag + a);
+            for (K m2 = m & (m - 1); m2; m2 &= m2 - 1) e += __ldg(p.G + a * norb + lowbit(m2));
+        }
+        const double hii = Eref + e;
+#pragma unroll
+        for (int v = 0; v < 8; v++) {
+            if (v >= R) break;
+            double num2;
+            if constexpr (CPLX) {
+                const double re = __longlong_as_double((long long)slot[KW + 2 * v]);
+                const double im = __longlong_as_double((long long)slot[KW + 1 + 2 * v]);
+                num2 = re * re + im * im;
+            } else {
+                const double num = __longlong_as_double((long long)slot[KW + v]);
+                num2 = num * num;
+            }
+            acc[v] += num2 / (E0[v] - hii);
+        }
+    });
+    __syncwarp();
+#pragma unroll
+    for (int v = 0; v < 8; v++) {
+        if (v >= R) break;
+        double x = acc[v];
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if ((threadIdx.x & 31) == 0) atomicAdd(out + v, x);
     }
 }
 
@@ -948,7 +999,7 @@ template <typename T>
 __global__ void k_pt2_setup(int norb, int dmax, uint64_t ref_lo, uint64_t ref_hi, uint64_t ref_w2, const T *__restrict__ h_so,
                             const T *__restrict__ jd, const T *__restrict__ kd, double *__restrict__ G,
                             double *__restrict__ fdiag, double *__restrict__ Eref, double *__restrict__ fix_scale,
-                            long long *__restrict__ fix, double *__restrict__ rest)
+                            long long *__restrict__ fix)
 {
     __shared__ unsigned long long s_max[2];   // largest |F| and |G|, as bits (ordered like the values)
     if (threadIdx.x < 2) s_max[threadIdx.x] = 0ull;
@@ -968,20 +1019,15 @@ __global__ void k_pt2_setup(int norb, int dmax, uint64_t ref_lo, uint64_t ref_hi
     }
     __syncthreads();
     // F and G as integers: the largest power of two that keeps any sum of them below 2^62 (the
-    // terms of dmax orbitals and of their pairs).  Integrals whose sums overflow FP64 give NaN.
+    // terms of dmax orbitals and of their pairs)
     const double d = max(dmax, 2);
     const double bound = d * __longlong_as_double((long long)s_max[0]) +
                          0.5 * d * (d - 1.0) * __longlong_as_double((long long)s_max[1]);
     int ex = 0;
     frexp(bound, &ex);   // bound < 2^ex
-    const double scale = bound <= 1.7976931348623157e308 ? ldexp(1.0, min(62 - ex, 1000)) : nan(""), unit = 1.0 / scale;
-    auto split = [&](double x, int at) {
-        const double u = x * scale;
-        fix[at] = llrint(u);
-        rest[at] = (u - (double)fix[at]) * unit;   // exact: u has 53 bits, and none left from 2^53 on
-    };
-    for (int t = threadIdx.x; t < norb; t += blockDim.x) split(fdiag[t], t);
-    for (int t = threadIdx.x; t < norb * norb; t += blockDim.x) split(G[t], norb + t);
+    const double scale = bound <= 1.7976931348623157e308 ? ldexp(1.0, min(62 - ex, 1000)) : nan("");
+    for (int t = threadIdx.x; t < norb; t += blockDim.x) fix[t] = llrint(fdiag[t] * scale);
+    for (int t = threadIdx.x; t < norb * norb; t += blockDim.x) fix[norb + t] = llrint(G[t] * scale);
     if (threadIdx.x == 0) {
         double e = 0.0;
         for (W3 m = ref; m; m &= m - 1) {
@@ -991,7 +1037,7 @@ __global__ void k_pt2_setup(int norb, int dmax, uint64_t ref_lo, uint64_t ref_hi
         }
         *Eref = e;
         fix_scale[0] = scale;
-        fix_scale[1] = unit > ldexp(fabs(e), -56) ? 1.0 : 0.0;
+        fix_scale[1] = 1.0 / scale <= ldexp(fabs(e), -56) ? 0.0 : 1.0;   // (1 for NaN)
     }
 }
 
@@ -1062,7 +1108,7 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
         if (tab2) cudaFree(tab2);
         if (bnd_free) cudaFree(bnd_free);
     };
-    const size_t nsmall = (size_t)R * 3 + 3 * ((size_t)norb * norb + norb) + 3 + 2;
+    const size_t nsmall = (size_t)R * 3 + 2 * ((size_t)norb * norb + norb) + 3 + 2;
     if (cudaMalloc(&S, sizeof(double) * SC * std::max<int64_t>(1, M) * R) != cudaSuccess ||
         cudaMalloc(&small, sizeof(double) * nsmall) != cudaSuccess) {
         cleanup();
@@ -1071,8 +1117,7 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
     double *dE0 = small, *outW = small + R, *outP = small + 2 * R, *G = small + 3 * R, *fdiag = G + norb * norb,
            *Eref = fdiag + norb;
     double *fix_scale = Eref + 1;
-    double *rest = fix_scale + 2;
-    long long *fix = reinterpret_cast<long long *>(rest + norb * norb + norb);
+    long long *fix = reinterpret_cast<long long *>(fix_scale + 2);
     unsigned long long *count = reinterpret_cast<unsigned long long *>(fix + norb * norb + norb);
     int *flag = reinterpret_cast<int *>(count + 1);
     if (sci_cuda_check(ctx, cudaMemsetAsync(small, 0, sizeof(double) * nsmall, st), "enpt2 memset") ||
@@ -1096,10 +1141,10 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
     const int dmax = 2 * (ctx->spinors ? std::min(ctx->N, n - ctx->N) : std::min(na, n - na) + std::min(nb, n - nb));
     if constexpr (SPIN)
         k_pt2_setup<zdbl><<<1, 256, 0, st>>>(norb, dmax, ctx->ref, ctx->ref_hi, ctx->ref_w2, (const zdbl *)ctx->h_so,
-                                             (const zdbl *)ctx->jd, (const zdbl *)ctx->kd, G, fdiag, Eref, fix_scale, fix, rest);
+                                             (const zdbl *)ctx->jd, (const zdbl *)ctx->kd, G, fdiag, Eref, fix_scale, fix);
     else
         k_pt2_setup<double><<<1, 256, 0, st>>>(norb, dmax, ctx->ref, ctx->ref_hi, ctx->ref_w2, (const double *)ctx->h_so,
-                                               (const double *)ctx->jd, (const double *)ctx->kd, G, fdiag, Eref, fix_scale, fix, rest);
+                                               (const double *)ctx->jd, (const double *)ctx->kd, G, fdiag, Eref, fix_scale, fix);
     // the table: capacity a power of two within the budget
     const size_t slot = sizeof(uint64_t) * SW;
     uint64_t cap = 1ull << 8;  // at least 256 entries
@@ -1148,7 +1193,7 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
     }
     p.n = n, p.norb = norb, p.na = na, p.nb = nb, p.ref = ctx->ref, p.ref_hi = ctx->ref_hi, p.ref_w2 = ctx->ref_w2;
     p.tab = (const double *)ctx->tab, p.fref = (const double *)ctx->fref, p.g_so = (const double *)ctx->g_so;
-    p.Eref = Eref, p.fix_scale = fix_scale, p.fix = fix, p.rest = rest;
+    p.fdiag = fdiag, p.G = G, p.Eref = Eref, p.fix_scale = fix_scale, p.fix = fix;
     p.tab2 = tab2, p.mask = cap - 1, p.count = count, p.flag = flag;
     p.limit = (unsigned long long)(0.85 * (double)cap);
     p.eps = eps;
@@ -1205,13 +1250,19 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
                 k_pt2_gen<R, KW><<<blocks, kThreads, 0, st>>>(ctx->keys, M, C, p, b, t);
         }
         if (sci_cuda_check(ctx, cudaEventRecord(ev[2], st), "enpt2 event")) return SCI_ERR_CUDA;
-        if (eval)
-            keval<<<grid_for((int64_t)std::min<uint64_t>(cap, 1ull << 40)), kThreads, eval_smem, st>>>(p, cap, dE0, outW);
+        const int grid = grid_for((int64_t)std::min<uint64_t>(cap, 1ull << 40));
+        if (eval) keval<<<grid, kThreads, eval_smem, st>>>(p, cap, dE0, outW);
         unsigned long long hc[2] = {0, 0};
         if (sci_cuda_check(ctx, cudaEventRecord(ev[3], st), "enpt2 event") ||
             sci_cuda_check(ctx, cudaMemcpyAsync(hc, count, sizeof(hc), cudaMemcpyDeviceToHost, st), "enpt2 flag") ||
             sci_cuda_check(ctx, cudaStreamSynchronize(st), "enpt2 pass"))
             return SCI_ERR_CUDA;
+        if (hc[1] >> 32) {   // flag[1]: the evaluation left the table to the FP64 sums
+            k_pt2_eval64<SPIN, KW><<<grid, kThreads, 0, st>>>(p, cap, R, SW, dE0, outW);
+            if (sci_cuda_check(ctx, cudaEventRecord(ev[3], st), "enpt2 event") ||
+                sci_cuda_check(ctx, cudaStreamSynchronize(st), "enpt2 pass"))
+                return SCI_ERR_CUDA;
+        }
         float a = 0.f, g = 0.f, e = 0.f;
         cudaEventElapsedTime(&a, ev[0], ev[1]);
         cudaEventElapsedTime(&g, ev[1], ev[2]);
