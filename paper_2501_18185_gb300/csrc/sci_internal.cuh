@@ -84,6 +84,7 @@ struct RefW {
 // up to 4,489 (140 spin-orbitals) 25.8 ms at 2048, 20.2 ms at 512; a space whose buckets
 // stay below 512 (30 orbitals, up to 441) is unchanged, and tiling it at 256 costs 2%.
 constexpr int kTileBucket = 512;
+constexpr int kSMs = 152;           // of a GB300: what launch sizes and window rows are set by
 constexpr int kSortBucket = 64;     // buckets of at most this many members go through the sorted kernel
 constexpr int kSmallBucket = 4;     // ... and of at most this many through the register kernel
 constexpr int kTileRows = 256;      // rows of a tile of the tiled kernel (one per thread)

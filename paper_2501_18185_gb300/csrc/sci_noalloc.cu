@@ -103,7 +103,7 @@ int grid_for(int64_t n)
 {
     int64_t g = (n + 255) / 256;
     if (g < 1) g = 1;
-    if (g > 152 * 32) g = 152 * 32;
+    if (g > sci::kSMs * 32) g = sci::kSMs * 32;
     return (int)g;
 }
 

@@ -1083,7 +1083,7 @@ __global__ void k_pt2_bounds_ab(int n, const double *__restrict__ T, double *__r
 
 int grid_for(int64_t n)
 {
-    return (int)std::max<int64_t>(1, std::min<int64_t>((n + kThreads - 1) / kThreads, 152 * 8));
+    return (int)std::max<int64_t>(1, std::min<int64_t>((n + kThreads - 1) / kThreads, sci::kSMs * 8));
 }
 
 // SPIN: complex spinor mode (C is [M][R] complex128); otherwise real spin-orbital mode.
@@ -1242,7 +1242,7 @@ int pt2_run(sci_ctx *ctx, const double *C, const double *E0h, double eps, size_t
             sci_cuda_check(ctx, cudaEventRecord(ev[1], st), "enpt2 event"))
             return SCI_ERR_CUDA;
         if (M > 0) {
-            const unsigned blocks = (unsigned)std::min<int64_t>((M + kWarps - 1) / kWarps, 152 * 16);
+            const unsigned blocks = (unsigned)std::min<int64_t>((M + kWarps - 1) / kWarps, sci::kSMs * 16);
             if constexpr (SPIN)
                 k_pt2_gen_z<R, KW><<<blocks, kThreads, 0, st>>>(ctx->keys, M, reinterpret_cast<const zdbl *>(C), p, b,
                                                                t);

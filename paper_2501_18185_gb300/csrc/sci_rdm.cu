@@ -591,7 +591,7 @@ template <typename TC> __global__ void __launch_bounds__(kThreads) k_rdm_expand2
 int grid_for(int64_t n)
 {
     const int64_t b = (n + kThreads - 1) / kThreads;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(b, 152 * 16));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(b, sci::kSMs * 16));
 }
 
 template <typename TC> struct Walk {
@@ -685,7 +685,7 @@ int rdm_tables(sci_ctx *ctx, const TC *C, int nvec, const double *wk_dev, bool w
     // window rows of the large buckets: short windows where there are few (shared memory, and
     // with it the CTAs per SM, is the largest bucket's: 441 members at 30 orbitals;
     // 1.47M entries of buckets above 64: 546 us at 768 rows, 491 at 256)
-    const int CH = ctx->split2.above[sci::kSortBucket] / 768 >= 152 * 16 ? 768 : 256;
+    const int CH = ctx->split2.above[sci::kSortBucket] / 768 >= sci::kSMs * 16 ? 768 : 256;
     auto stage_bytes = [&](int nv) {
         return (size_t)(CH + ctx->maxb2) * (nv * sizeof(TC) + 2 * sizeof(uint32_t));
     };
@@ -708,7 +708,7 @@ int rdm_tables(sci_ctx *ctx, const TC *C, int nvec, const double *wk_dev, bool w
         return SCI_ERR_CUDA;
     for (int v0 = 0; v0 < nvec; v0 += kv) {
         const int nv = std::min(kv, nvec - v0);
-        kd<<<std::min(grid_for(ctx->M), 152 * 7), kThreads, diag_smem, ctx->stream>>>(ctx->keys, ctx->M, norb, ref_words(ctx), C, nvec, v0,
+        kd<<<std::min(grid_for(ctx->M), sci::kSMs * 7), kThreads, diag_smem, ctx->stream>>>(ctx->keys, ctx->M, norb, ref_words(ctx), C, nvec, v0,
                                                                    nv, wk_dev, Wt, D, DD);
         const Walk<TC> wlk{C, nvec, v0, wk_dev, A, Bc, with_two && ctx->e2 > 0 ? dT : nullptr, CH, stage_bytes(nv), tr, bb_off};
         int rc = SCI_OK;

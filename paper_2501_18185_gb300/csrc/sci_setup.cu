@@ -521,7 +521,7 @@ int grid_for(int64_t n, int threads = 256)
 {
     int64_t g = (n + threads - 1) / threads;
     if (g < 1) g = 1;
-    if (g > 152 * 64) g = 152 * 64;
+    if (g > sci::kSMs * 64) g = sci::kSMs * 64;
     return (int)g;
 }
 

@@ -390,11 +390,11 @@ template <class P, int NV> constexpr int wide_ctas()
     constexpr int c = min_ctas<P, NV>();
     return f32_wide<P, NV>() ? c : c == 8 ? 6 : c == 6 ? 5 : c;
 }
-// Window rows of that walk: `rows` or 512 when they give kWindowsWanted windows (two for
-// every resident CTA), else 256 (60k space: 85 windows of 768 rows 227 us, 254 of 256 rows 148
+// Window rows of that walk: `rows` or 512 when they give kWindowsWanted windows, 16 an SM, three
+// to four for each of its 4 to 6 resident CTAs, else 256 (a measured line: 60k space: 85 windows of 768 rows 227 us, 254 of 256 rows 148
 // us; 40 orbitals, two vectors: 1,188 of 768 rows 1.21 ms, 3,563 of 256 1.14 ms; with 6,645
 // windows of 768 rows, on the 2M space, 256 rows cost 3%).
-constexpr int64_t kWindowsWanted = 152 * 16;
+constexpr int64_t kWindowsWanted = sci::kSMs * 16;
 inline int window_rows(int64_t entries, int rows)
 {
     for (int r : {rows, 512})
@@ -1164,7 +1164,7 @@ int grid_for(int64_t n, int threads = kThreads)
 {
     int64_t g = (n + threads - 1) / threads;
     if (g < 1) g = 1;
-    if (g > 152 * 32) g = 152 * 32;
+    if (g > sci::kSMs * 32) g = sci::kSMs * 32;
     return (int)g;
 }
 
@@ -1235,7 +1235,7 @@ int launch_tiled(sci_ctx *ctx, const Tabs &T, const sci::Split &sp, const typena
     // us unsplit, 121.  Wide vector groups pay for each split with as many atomics per row
     // and stop at one wave (56 orbitals, 8 vectors: 6.43 ms at one, 6.84 at four).
     int nsplit = 1;
-    const int64_t ctas = 152 * (NV * sizeof(typename P::SC) >= sci::kWideRowBytes ? 8 : 32);
+    const int64_t ctas = sci::kSMs * (NV * sizeof(typename P::SC) >= sci::kWideRowBytes ? 8 : 32);
     if (!ST && sp.ntiles < ctas) {
         const int64_t want = (ctas + sp.ntiles - 1) / sp.ntiles;
         const int cols = (int)std::max<int64_t>(64, ((ctx->maxb2 + want - 1) / want + 31) & ~(int64_t)31);
