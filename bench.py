@@ -183,6 +183,42 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
+def kernels_per_sigma(H, C, S, prec) -> int:
+    """Kernels of the library in one product: the kernel nodes of a CUDA graph captured from the
+    call (all of them are the library's; one product has no copies).  The double excitations
+    are several launches, by bucket size; three kernels (init, doubles, singles) is the least."""
+    import ctypes
+
+    import torch
+
+    old, st = H.stream, torch.cuda.Stream()
+    try:
+        with open("/proc/self/maps") as f:
+            path = next(line.split()[-1] for line in f if "libcudart" in line)
+        rt = ctypes.CDLL(path)
+        torch.cuda.synchronize()
+        H.set_stream(st)
+        graph = torch.cuda.CUDAGraph(keep_graph=True)
+        with torch.cuda.graph(graph, stream=st):
+            H.sigma(C, out=S, prec=prec)
+        g, n = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t()
+        if rt.cudaGraphGetNodes(g, None, ctypes.byref(n)):
+            return 3
+        nodes = (ctypes.c_void_p * n.value)()
+        if rt.cudaGraphGetNodes(g, nodes, ctypes.byref(n)):
+            return 3
+        kind, count = ctypes.c_int(), 0
+        for node in nodes:
+            if rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)):
+                return 3
+            count += kind.value == 0          # cudaGraphNodeTypeKernel
+        return max(count, 3)
+    except (OSError, StopIteration, AttributeError, TypeError, RuntimeError):
+        return 3
+    finally:
+        H.set_stream(old)
+
+
 def cpu_model() -> str:
     """The host CPU as /proc/cpuinfo names it (model name, or the Arm implementer and part
     numbers when there is no model name)."""
@@ -1156,6 +1192,7 @@ def main():
                              "singles": statistics.mean(k[2] for k in o_kern)}}
     sci.sci_profile(H.ctx, False)
     H.sync_status()
+    kernels = kernels_per_sigma(H, C, S, prec)
 
     total_ms = max_over_ranks(sum(step_ms), dist, dev)
     ms = total_ms / args.steps
@@ -1257,8 +1294,7 @@ def main():
                        **({"rank0_rows": list(split.ranges[0]), "split_setup_s": round(split_setup_s, 3)}
                           if split is not None else {})},
             "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": nbytes, "d2h_bytes_per_step": nbytes_out},
-            "gpu_launches": args.steps * (1 + {"f64": 2, "ds": 4, "f32": 3}[args.prec]
-                                          * ((nv + 7) // 8 if not w.ints.complex_ else (nv + 3) // 4)),
+            "gpu_launches": args.steps * kernels,
             "roofline": roof, "cpu_baseline": cpu, "clocks": clocks, "prec": args.prec,
             "other_prec": variant, "pipe_peaks": pp, "davidson": dav, "rdm": rdm, "batch": batch, "pt2": pt2,
             "spinor": spinor, "rowsplit": rowsplit, "deterministic": determ, "two_word": two_word}
