@@ -959,7 +959,7 @@ void free_ints(sci_ctx *ctx)
     free_held(ctx, ctx->h_so);
     free_held(ctx, ctx->jd);
     free_held(ctx, ctx->kd);
-    free_held(ctx, ctx->gd);
+    ctx->gd = nullptr;   // part of kd
     free_held(ctx, ctx->g_so);
     free_held(ctx, ctx->tab);
     free_held(ctx, ctx->tab32);
@@ -1322,8 +1322,8 @@ int set_ints(sci_ctx *ctx, int scalar, int mode, int n, const void *h, const voi
     int norb = ctx->norb;
     SCI_CK(alloc_held(ctx, &ctx->h_so, (size_t)norb * norb * sb));
     SCI_CK(alloc_held(ctx, &ctx->jd, (size_t)norb * norb * sb));
-    SCI_CK(alloc_held(ctx, &ctx->kd, (size_t)norb * norb * sb));
-    SCI_CK(alloc_held(ctx, (void **)&ctx->gd, (size_t)norb * norb * 8));
+    SCI_CK(alloc_held(ctx, &ctx->kd, (size_t)norb * norb * (sb + 8)));   // and gd, which saves an allocation
+    ctx->gd = reinterpret_cast<double *>((char *)ctx->kd + (size_t)norb * norb * sb);
     SCI_CK(alloc_held(ctx, &ctx->g_so, (size_t)norb * norb * norb * sb));
     OrbMap om{n, ctx->spinors};
     int64_t n3 = (int64_t)norb * norb * norb;

@@ -423,24 +423,27 @@ template <class P, int NV> constexpr int sort_from(bool small_table)
     if (!P::kFp64) return kSortBucket + 1;
     return NV == 1 && sizeof(typename P::SC) == sizeof(double) && !small_table ? 33 : kSmallBucket + 1;
 }
-// Entries of the buckets of at most kSortBucket members up to which the paired-FP32 and
-// FP32-storage launches take them in the aligned walk of the larger ones instead of by size: a
-// launch costs about 2 us, and these policies gain less by size than FP64 does.  Two
-// paired-FP32 vectors, the product: 30 orbitals, 1,000 determinants (76k entries) 70 us by size,
-// 43 in one walk; 3,000 (118k) 75, 45; full CI of 8 orbitals (137k) 51, 45; 40 orbitals, M =
-// 60k, one vector (922k) 209, 228; FP32 storage at 8 vectors, 221k entries 51, 60.
+// Table entries up to which the paired-FP32 and FP32-storage launches take the buckets of at most
+// kSortBucket members in the aligned walk of the larger ones instead of by size: a launch costs
+// about 2 us, and these policies gain less by size than FP64 does.  Two paired-FP32 vectors, the
+// product: 30 orbitals, 1,000 determinants (76k entries) 70 us by size, 43 in one walk; 3,000 (118k)
+// 75, 45; full CI of 8 orbitals (137k) 51, 45; 40 orbitals, M = 60k, one vector (1.4M) 209, 228; FP32
+// storage at 8 vectors, 221k entries 51, 60; 100 orbitals, 360k entries most of them in tiles, the
+// deterministic mode at three vectors 2.25 ms, 2.41.
 constexpr int64_t kFewEntries = 200'000;
-// ... and in a row range in FP32 storage, when the space has larger buckets too: a short range
-// owns few of a bucket's rows, and the launches by size stage and sort the others all the same.
+// ... and in a row range in FP32 storage, when the space has larger buckets too, by the entries
+// left to them: a short range owns few of a bucket's rows, and the launches by size stage and sort
+// the others all the same.
 // M = 400k, a 64th of the rows, 8 vectors (1.4M entries): 153 us by size, 140; M = 60k, an eighth,
 // one vector (2.5M): 91, 84; M = 400k, an eighth, one vector (6.5M): 143, 162.  (Without larger
 // buckets the windows are too short for the rows they own: full CI of 10 orbitals, a 64th, 8
 // vectors, 221k entries: 51, 60.)
 constexpr int64_t kFewRangeEntries = 3'000'000;
-template <class P, bool RANGED> constexpr int64_t few_entries(bool larger)
+// b: the end of the tiles, large: of the buckets above kSortBucket members
+template <class P, bool RANGED> constexpr bool in_one_walk(int64_t entries, int64_t b, int64_t large)
 {
-    if (P::kFp64) return 0;
-    return RANGED && !P::kSplit && larger ? kFewRangeEntries : kFewEntries;
+    if (P::kFp64) return false;
+    return entries <= kFewEntries || (RANGED && !P::kSplit && large > b && entries - large <= kFewRangeEntries);
 }
 // The tiled walk takes 32 columns at a time as a mask of doubles for complex FP64 (64
 // spinors, M = 500k: 1.43 -> 1.25 ms) and one FP64 vector (70 orbitals, M = 120k: doubles
@@ -1287,7 +1290,7 @@ int launch_doubles(sci_ctx *ctx, const Tabs &T, const typename P::TT *tab, const
     // ones at so, the aligned ones of five members and more at sm
     const int64_t *above = T.ts->above;
     const int64_t b = sp.big, large = std::max(b, above[kSortBucket]);
-    const int64_t m = T.e2 - large <= few_entries<P, RG>(large > b) ? T.e2 : large;
+    const int64_t m = in_one_walk<P, RG>(T.e2, b, large) ? T.e2 : large;
     constexpr int lowest = sort_from<P, NV>(true);
     const int from = sort_from<P, NV>(ctx->tab_elems * (int64_t)sizeof(typename P::TT) <= kSmallTable);
     const int64_t sm = lowest <= kSmallBucket ? T.e2 : std::max(m, above[kSmallBucket]);
