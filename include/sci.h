@@ -193,7 +193,7 @@ int sci_set_row_range(sci_ctx *ctx, int64_t row_begin, int64_t row_end);
  * the deterministic mode stays bit for bit reproducible at a fixed threshold.  Density
  * matrices (sci_rdm12) keep whole-bucket staging and return SCI_ERR_OVERFLOW for a bucket
  * that does not fit.  A threshold above what the window kernels can stage returns
- * SCI_ERR_OVERFLOW and keeps the previous one.  Synchronous (waits for the context
+ * SCI_ERR_OVERFLOW.  A call that fails, for this or any other reason, keeps the previous one.  Synchronous (waits for the context
  * stream; rebuilds the tile lists of the list and of a row range).  Errors: SCI_ERR_ARG
  * for members outside [0, 65535]. */
 int sci_set_tile_threshold(sci_ctx *ctx, int members);
